@@ -192,7 +192,8 @@ def reference_arm(args, w):
 # GPU leg
 # --------------------------------------------------------------------------
 
-KERNEL_SOURCES = ("svd_warp.cuh", "tnrc_device.cuh", "traj.cu")
+KERNEL_SOURCES = ("svd_fx.cuh", "tnrc_device.cuh", "traj_impl.cuh")
+KERNEL_HEADERS = ("fx.cuh", "svd_warp.cuh")   # what they include, hashed where present
 
 
 def recorded_counters(workload):
@@ -211,8 +212,9 @@ def recorded_counters(workload):
         if sep and key.strip() and " " not in key.strip():
             rec[key.strip()] = val.strip()
     h = hashlib.sha256()
-    for name in KERNEL_SOURCES:
-        with open(os.path.join(ROOT, "paper_2603_03639_gb300", "csrc", name), "rb") as f:
+    csrc = os.path.join(ROOT, "paper_2603_03639_gb300", "csrc")
+    for name in KERNEL_SOURCES + tuple(n for n in KERNEL_HEADERS if os.path.exists(os.path.join(csrc, n))):
+        with open(os.path.join(csrc, name), "rb") as f:
             h.update(f.read())
     if rec.get("workload") != workload or rec.get("kernel_sources_sha256") != h.hexdigest():
         return None

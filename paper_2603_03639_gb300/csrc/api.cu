@@ -116,6 +116,7 @@ tnrc::TrajParams traj_params(tnrc_ctx* ctx, bool grad) {
   tp.want_grad = grad ? 1 : 0;
   tp.warps = P.warps;
   tp.slab_elems = P.slab_elems;
+  tp.cta_slab_elems = tp.warps * tp.slab_elems;
   tp.min_blocks = P.d == 4 ? 1 : P.min_blocks;
   tp.phys_dim = P.d;
   tp.full.L = P.L;
@@ -522,6 +523,7 @@ tnrc_status tnrc_fidelity_grad_plain(tnrc_ctx* ctx, double* F, double* grad) {
   tnrc::TrajParams tp = traj_params(ctx, true);
   tp.warps = 2;   // the environment launch runs two warps; the others one
   tp.slab_elems = P.slab_elems;   // the batched launch's slab: the same bonds go as pairs
+  tp.cta_slab_elems = tp.warps * tp.slab_elems;
   tp.warp_scratch = reinterpret_cast<double2*>(ctx->plain + off_scr);
   tp.env_scratch = reinterpret_cast<double2*>(ctx->plain + off_env);
   const size_t smem = tnrc_traj_smem(2, tp.slab_elems);

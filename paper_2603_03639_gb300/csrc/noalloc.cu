@@ -218,6 +218,7 @@ extern "C" tnrc_status tnrc_fidelity_static(const tnrc_problem* pb, const tnrc_m
   tp.want_grad = 0;
   tp.warps = warps;
   tp.slab_elems = slab;
+  tp.cta_slab_elems = tp.warps * tp.slab_elems;
   tp.min_blocks = 1;
   tp.phys_dim = d;
   tp.full.L = L;

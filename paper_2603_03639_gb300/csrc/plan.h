@@ -125,11 +125,18 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
     P.site_off = Y.site_off;
     P.L = Y.L;
   }
-  int maxb = 0;
-  for (int par = 0; par < 2; ++par) maxb = std::max(maxb, (N - 1 - par + 1) / 2);
-  P.warps = std::max(2, std::min(tnrc::kWarps, maxb));
+  // all warps even where a layer has fewer bonds: they share the environment
+  // sweeps and the large updates
+  P.warps = tnrc::kWarps;
   if (pb->warps_per_cta < 0 || pb->warps_per_cta == 1 || pb->warps_per_cta > tnrc::kWarps) return false;
   if (pb->ctas_per_sm < 0 || pb->ctas_per_sm > 4) return false;
+  // two CTAs of half the warps once the trajectories fill them: each CTA's
+  // serial stretches (environment sweeps, layer barriers) then run beside the
+  // other's updates (cnot50 near the solution, 304 trajectories: 479 ms as 8
+  // x 1, 386 ms as 4 x 2; with 152 trajectories of ghz30, 172 and 233 ms)
+  const bool two = pb->warps_per_cta == 0 && pb->ctas_per_sm == 0 && P.warps == tnrc::kWarps &&
+                   2 * T >= 3ll * n_sm;
+  if (two) P.warps = tnrc::kWarps / 2;
   if (pb->warps_per_cta > 0) P.warps = pb->warps_per_cta;
   if (const char* e = getenv("TNRC_WARPS")) {
     const int w = atoi(e);
@@ -138,7 +145,7 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
   // the register file holds 8 warps of the 255-register build per SM and 16 of
   // the 128-register build; more than 8 warps per SM select the latter
   const int ctas_per_sm =
-      std::max(1, std::min(pb->ctas_per_sm > 0 ? pb->ctas_per_sm : 1, (P.d == 4 ? 1 : 2) * tnrc::kWarps / P.warps));
+      std::max(1, std::min(pb->ctas_per_sm > 0 ? pb->ctas_per_sm : two ? 2 : 1, (P.d == 4 ? 1 : 2) * tnrc::kWarps / P.warps));
   P.min_blocks = (P.warps * ctas_per_sm > tnrc::kWarps) ? 2 : 1;
   // each warp's shared slab holds theta^dagger up to slab_elems complex values
   // (wider thetas use global scratch): split what the resident CTAs of an SM

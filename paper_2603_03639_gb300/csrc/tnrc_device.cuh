@@ -21,8 +21,8 @@ constexpr int kMaxSweeps = 60;              // Jacobi sweep limit
 constexpr double kZeroFloor = 1e-13;        // relative numerical-zero level of singular values
 constexpr double kJacobiZero = 5e-15;       // columns below this x ||theta||_F are left alone
 constexpr double kJacobiQuad = 1e-20;       // |<a,b>|^2 / (|a|^2 |b|^2) of a rotation that counts as
-                                            // large: a sweep with none is the last (quadratic convergence)
-constexpr int kRowQrMinRank = 8;            // second QR of R^dagger from this rank on, when n >= 2.5 r
+                                            // large in warp_jacobi: a sweep with none is the last
+                                            // (quadratic convergence)
 
 // device status bits (OR-ed into *status)
 constexpr int kStatusNoConverge = 1;
@@ -100,6 +100,7 @@ struct TrajParams {
   int min_blocks;              // register budget of the launch: 1 = up to 8 warps per SM
                                // (255 registers), 2 = up to 16 warps per SM (128 registers)
   int slab_elems;              // complex elements of each warp's shared slab
+  int cta_slab_elems;          // of all warps' slabs together (contiguous)
   Lay full;                    // capacities min(2^i, 2^(N-i), chi)
   int packed_history;          // keep the forward history packed (no recomputation)
   long long history_cap;       // upper bound on a CTA's packed-history bytes
