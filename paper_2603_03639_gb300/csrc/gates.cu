@@ -1,6 +1,6 @@
 // Layer gate table of the truncated TEBD layers, and the noise realisations.
 //
-// layer_gate_kernel: one thread per (sample s, truncated layer l, bond b of
+// layer_gate_kernel: eight lanes per (sample s, truncated layer l, bond b of
 // that layer).  The layer's gate on bond b is a product of factors
 // exp(-i tau h_f) (time order f = 1..F), each h_f Hermitian and linear in the
 // controls it contains:
@@ -25,110 +25,145 @@
 
 namespace tnrc {
 
-__device__ __forceinline__ void herm_rotate(double2 (&h)[16], double2 (&V)[16], int p, int q) {
-  const double2 z = h[p * 4 + q];
-  const double az2 = cabs2(z);
-  if (az2 == 0.0) return;
-  const double inv = rsqrt(az2);
-  const double2 ph = make_double2(z.x * inv, z.y * inv);  // e^{i phi}
-  const double a = h[p * 4 + p].x, d = h[q * 4 + q].x;
-  const double zeta = (d - a) * 0.5 * inv;
-  double t;
-  if (fabs(zeta) > 1e150)
-    t = 0.5 / zeta;
-  else
-    t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
-  const double c = rsqrt(fma(t, t, 1.0));
-  const double s = c * t;
-  // U = [[c, s], [-s e^{-i phi}, c e^{-i phi}]] on (p, q):  h <- U^dag h U,  V <- V U
-  const double2 u00 = make_double2(c, 0.0), u01 = make_double2(s, 0.0);
-  const double2 u10 = make_double2(-s * ph.x, s * ph.y);
-  const double2 u11 = make_double2(c * ph.x, -c * ph.y);
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {  // columns
-    const double2 hp = h[r * 4 + p], hq = h[r * 4 + q];
-    double2 np = cmul(hp, u00), nq = cmul(hp, u01);
-    cfma(np, hq, u10);
-    cfma(nq, hq, u11);
-    h[r * 4 + p] = np;
-    h[r * 4 + q] = nq;
-    const double2 vp = V[r * 4 + p], vq = V[r * 4 + q];
-    double2 wp = cmul(vp, u00), wq = cmul(vp, u01);
-    cfma(wp, vq, u10);
-    cfma(wq, vq, u11);
-    V[r * 4 + p] = wp;
-    V[r * 4 + q] = wq;
-  }
-#pragma unroll
-  for (int cidx = 0; cidx < 4; ++cidx) {  // rows
-    const double2 hp = h[p * 4 + cidx], hq = h[q * 4 + cidx];
-    double2 np = make_double2(0.0, 0.0), nq = make_double2(0.0, 0.0);
-    cfmac(np, u00, hp);
-    cfmac(np, u10, hq);
-    cfmac(nq, u01, hp);
-    cfmac(nq, u11, hq);
-    h[p * 4 + cidx] = np;
-    h[q * 4 + cidx] = nq;
-  }
-  h[p * 4 + q] = make_double2(0.0, 0.0);
-  h[q * 4 + p] = make_double2(0.0, 0.0);
-  h[p * 4 + p].y = 0.0;
-  h[q * 4 + q].y = 0.0;
+// Eight lanes work on one record: two factors (later: two controls) at a time,
+// each by four lanes, lane r holding row r of its 4 x 4 matrices.  One thread
+// per record was a chain of FP64 instructions of 0.9 ms (64 cycles each, square
+// roots and divisions 600) whatever the number of records, half of a small
+// evaluation: the smallest call went from 1.63 to 1.05 ms.  The FP64
+// instructions per record stay about the same (the lanes share them).
+constexpr int kRecLanes = 8;
+constexpr int kGateThreads = 64;
+constexpr int kMaxFactors = 5;
+
+__device__ __forceinline__ double2 shfl4(double2 v, int src) {   // from lane src of the group of four
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src, 4), __shfl_sync(0xffffffffu, v.y, src, 4));
 }
 
-// Hermitian 4x4 eigendecomposition h = V diag(lam) V^dag by cyclic Jacobi
-// rotations; h is overwritten.  Returns false if it did not converge.
-__device__ bool herm_eig4(double2 (&h)[16], double2 (&V)[16], double (&lam)[4]) {
+// Cyclic Jacobi of the Hermitian 4 x 4 matrix whose row r is h: on return the
+// diagonal holds the eigenvalues and v is row r of V, h = V diag V^dagger.  A
+// round rotates two disjoint pairs (p, q), U = [[c, s], [-conj(s), c]]; the
+// angle is FP32 (each round still shrinks its off-diagonal entries by 1e-7),
+// the rotation unitary to FP64 rounding.  Returns false if it did not converge.
+__device__ bool herm_eig4_rows(double2 (&h)[4], double2 (&v)[4], int r) {
 #pragma unroll
-  for (int i = 0; i < 16; ++i) V[i] = make_double2((i % 5 == 0) ? 1.0 : 0.0, 0.0);
-  double scale2 = 0.0;
+  for (int c = 0; c < 4; ++c) v[c] = make_double2(c == r ? 1.0 : 0.0, 0.0);
+  double sc = 0.0;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) scale2 += cabs2(h[i]);
-  const double stop2 = 1e-32 * scale2;
+  for (int c = 0; c < 4; ++c) sc += cabs2(h[c]);
+  sc += __shfl_xor_sync(0xffffffffu, sc, 1, 4);
+  sc += __shfl_xor_sync(0xffffffffu, sc, 2, 4);
+  // 2^-e with 2^(2e) about sc: the FP32 angles see entries of order one
+  const int e2 = (__double2hiint(sc) >> 20) & 2047;
+  const double inv = __hiloint2double((1023 - ((e2 - 1023) >> 1)) << 20, 0);
   bool ok = false;
+#pragma unroll 1
   for (int sweep = 0; sweep < 30; ++sweep) {
-    double off2 = 0.0;
+    double off = 0.0;
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int c = 0; c < 4; ++c)
+      if (c != r) off += cabs2(h[c]);
+    off += __shfl_xor_sync(0xffffffffu, off, 1, 4);
+    off += __shfl_xor_sync(0xffffffffu, off, 2, 4);
+    ok = off <= 2e-32 * sc;
+    if (__all_sync(0xffffffffu, ok)) break;
 #pragma unroll
-      for (int q = p + 1; q < 4; ++q) off2 += cabs2(h[p * 4 + q]);
-    if (off2 <= stop2) {
-      ok = true;
-      break;
+    for (int rd = 0; rd < 3; ++rd) {
+      // partner of index i in round rd: i ^ 1, i ^ 2, i ^ 3
+      const int mate = r ^ (rd + 1);
+      const bool low = r < mate;
+      // z = h[p][q] (p < q), d = h[q][q] - h[p][p], the same in both lanes of a pair
+      double2 hm = h[0], hd = h[0];
+#pragma unroll
+      for (int c = 1; c < 4; ++c) {
+        if (c == mate) hm = h[c];
+        if (c == r) hd = h[c];
+      }
+      if (r == 0) hd = h[0];
+      const double other = __shfl_sync(0xffffffffu, hd.x, mate, 4);
+      const double2 z = shfl4(hm, low ? r : mate);
+      const float zx = (float)(z.x * inv), zy = (float)(z.y * inv);
+      const float z2 = fmaf(zx, zx, zy * zy);
+      float tx = 0.0f, ty = 0.0f;
+      if (z2 > 0.0f) {
+        const float d = (float)((low ? other - hd.x : hd.x - other) * inv);
+        const float iz = rsqrtf(z2), az = z2 * iz;
+        // tan = 2 |z| / (|d| + sqrt(d^2 + 4 |z|^2)), phase of z, sign of d
+        const float t = copysignf(2.0f * az * __fdividef(1.0f, fabsf(d) + sqrtf(fmaf(d, d, 4.0f * z2))), d);
+        tx = t * iz * zx;
+        ty = t * iz * zy;
+      }
+      // c = 1 / sqrt(1 + |t|^2) by one third-order step from FP32, s = c t
+      const double dx = tx, dy = ty;
+      const double w = fma(dx, dx, fma(dy, dy, 1.0));
+      const double y0 = (double)rsqrtf((float)w);
+      const double e = fma(-w * y0, y0, 1.0);
+      const double c = fma(y0 * e, fma(e, 0.375, 0.5), y0);
+      const double2 s = make_double2(c * dx, c * dy);
+      // columns of both pairs: (p, q) <- (c p - conj(s) q, s p + c q)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int p0 = rd == 0 ? 2 * k : k, q0 = p0 ^ (rd + 1);
+        const int a = p0 < q0 ? p0 : q0, b2 = p0 < q0 ? q0 : p0;
+        const double ck = __shfl_sync(0xffffffffu, c, a, 4);
+        const double2 sk = shfl4(s, a);
+        const double2 hp = h[a], hq = h[b2], vp = v[a], vq = v[b2];
+        double2 np = cscale(hp, ck), nq = cscale(hq, ck), wp = cscale(vp, ck), wq = cscale(vq, ck);
+        cfmac(np, make_double2(-sk.x, -sk.y), hq);
+        cfma(nq, sk, hp);
+        cfmac(wp, make_double2(-sk.x, -sk.y), vq);
+        cfma(wq, sk, vp);
+        h[a] = np;
+        h[b2] = nq;
+        v[a] = wp;
+        v[b2] = wq;
+      }
+      // rows: p <- c p - s q, q <- conj(s) p + c q
+      const double2 sr = low ? make_double2(-s.x, -s.y) : cconj(s);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const double2 o = shfl4(h[k], mate);
+        double2 nh = cscale(h[k], c);
+        cfma(nh, sr, o);
+        h[k] = nh;
+      }
+      // an entry of 1e-10 is zero now up to 1e-17 (the FP32 angle) and rounding
+      if (z2 <= 1e-20f) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k == mate) h[k] = make_double2(0.0, 0.0);
+      }
     }
-    herm_rotate(h, V, 0, 1);
-    herm_rotate(h, V, 2, 3);
-    herm_rotate(h, V, 0, 2);
-    herm_rotate(h, V, 1, 3);
-    herm_rotate(h, V, 0, 3);
-    herm_rotate(h, V, 1, 2);
   }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) lam[j] = h[j * 5].x;
   return ok;
 }
 
-// Generators in the bond basis |s_b s_{b+1}> (index 2 s_b + s_{b+1}), scaled by w:
-// 0: X (x) I, 1: Y (x) I, 2: I (x) X, 3: I (x) Y, 4: Z (x) Z.
-__device__ void generator4(int code, double w, double2 (&P)[16]) {
-#pragma unroll
-  for (int i = 0; i < 16; ++i) P[i] = make_double2(0.0, 0.0);
-  switch (code) {
-    case 0:
-      P[0 * 4 + 2].x = w; P[1 * 4 + 3].x = w; P[2 * 4 + 0].x = w; P[3 * 4 + 1].x = w;
-      break;
-    case 1:
-      P[0 * 4 + 2].y = -w; P[1 * 4 + 3].y = -w; P[2 * 4 + 0].y = w; P[3 * 4 + 1].y = w;
-      break;
-    case 2:
-      P[0 * 4 + 1].x = w; P[1 * 4 + 0].x = w; P[2 * 4 + 3].x = w; P[3 * 4 + 2].x = w;
-      break;
-    case 3:
-      P[0 * 4 + 1].y = -w; P[1 * 4 + 0].y = w; P[2 * 4 + 3].y = -w; P[3 * 4 + 2].y = w;
-      break;
-    default:
-      P[0].x = w; P[5].x = -w; P[10].x = -w; P[15].x = w;
-      break;
+// sin(x) / x, with sn = sin x known to about 1e-16
+__device__ __forceinline__ double sinc_of(double x, double sn) {
+  const double x2 = x * x;
+  if (x2 < 0.25) {   // Taylor series to x^14: the next term is below 1e-18
+    double p = -1.0 / 1307674368000.0;
+    p = fma(p, x2, 1.0 / 6227020800.0);
+    p = fma(p, x2, -1.0 / 39916800.0);
+    p = fma(p, x2, 1.0 / 362880.0);
+    p = fma(p, x2, -1.0 / 5040.0);
+    p = fma(p, x2, 1.0 / 120.0);
+    p = fma(p, x2, -1.0 / 6.0);
+    return fma(p, x2, 1.0);
+  }
+  return sn / x;
+}
+
+// Row i of a generator in the bond basis |s_b s_{b+1}> (index 2 s_b + s_{b+1}),
+// scaled by w: one entry, `val` in column `col`.  0: X (x) I, 1: Y (x) I,
+// 2: I (x) X, 3: I (x) Y, 4: Z (x) Z.
+__device__ __forceinline__ void generator_row(int code, double w, int i, int& col, double2& val) {
+  const int bit = code < 2 ? 2 : 1;
+  if (code == 4) {
+    col = i;
+    val = make_double2((i == 0 || i == 3) ? w : -w, 0.0);
+  } else {
+    col = i ^ bit;
+    val = (code & 1) ? make_double2(0.0, (i & bit) ? w : -w) : make_double2(w, 0.0);
   }
 }
 
@@ -146,54 +181,62 @@ struct LayerGateArgs {
 
 // factor kinds
 constexpr int kFBond = 0, kFInter = 1, kFXl = 2, kFYl = 3, kFXr = 4, kFYr = 5;
-constexpr int kMaxFactors = 5;
 
-__global__ void layer_gate_kernel(LayerGateArgs a) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)a.M * a.R) return;
+struct GateShared {                     // one record
+  double2 V[kMaxFactors][16], G[kMaxFactors][16], GE[kMaxFactors][16];
+  double2 T[2][16], Lt[16];
+};
+
+__global__ void __launch_bounds__(kGateThreads) layer_gate_kernel(LayerGateArgs a) {
+  __shared__ GateShared sh[kGateThreads / kRecLanes];
+  const int lane8 = threadIdx.x & (kRecLanes - 1), half = lane8 >> 2, r = lane8 & 3;
+  GateShared& S = sh[threadIdx.x / kRecLanes];
+  const long long total = (long long)a.M * a.R;
+  const long long idx0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kRecLanes;
+  const bool live = idx0 < total;
+  const long long idx = live ? idx0 : total - 1;   // idle groups repeat the last record and write nothing
   const int s = (int)(idx / a.R);
-  const int r = (int)(idx - (long long)s * a.R);
-  int lo = 0, hi = a.L;  // largest l with layer_off[l] <= r
+  const int rec = (int)(idx - (long long)s * a.R);
+  int lo = 0, hi = a.L;  // largest l with layer_off[l] <= rec
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if (a.layer_off[mid] <= r) lo = mid; else hi = mid;
+    if (a.layer_off[mid] <= rec) lo = mid; else hi = mid;
   }
   const int l = lo;
   const int parity = (l + a.first_parity) & 1;
-  const int b = parity + 2 * (r - a.layer_off[l]);
+  const int b = parity + 2 * (rec - a.layer_off[l]);
   const int N = a.N, nb = N - 1;
-  const int S = a.K * a.nsub;
+  const int St = a.K * a.nsub;
   const double dts = a.dt / a.nsub;
 
-  // the layer's factors on bond b, first in time first
-  int fk[kMaxFactors], fkind[kMaxFactors];
-  double ftau[kMaxFactors];
-  int nf = 0;
+  // the layer's factors on bond b, first in time first: kind, bin and duration of factor f
+  int nf, kind0 = kFBond, k0, k1;
+  double tau;
   if (a.order == 2) {
+    nf = 1;
     if (l & 1) {
-      fkind[nf] = kFBond; fk[nf] = ((l - 1) >> 1) / a.nsub; ftau[nf++] = dts;
-    } else if (l == 0) {
-      fkind[nf] = kFBond; fk[nf] = 0; ftau[nf++] = 0.5 * dts;
-    } else if (l == 2 * S) {
-      fkind[nf] = kFBond; fk[nf] = (S - 1) / a.nsub; ftau[nf++] = 0.5 * dts;
+      k0 = k1 = ((l - 1) >> 1) / a.nsub;
+      tau = dts;
     } else {
-      const int st = (l >> 1) - 1;
-      fkind[nf] = kFBond; fk[nf] = st / a.nsub; ftau[nf++] = 0.5 * dts;
-      fkind[nf] = kFBond; fk[nf] = (st + 1) / a.nsub; ftau[nf++] = 0.5 * dts;
+      const int st = (l >> 1) - 1;   // the half steps of steps st and st + 1, merged
+      tau = 0.5 * dts;
+      k0 = (l == 0 ? 0 : st) / a.nsub;
+      k1 = (l == 2 * St ? St - 1 : st + 1) / a.nsub;
+      if (l != 0 && l != 2 * St) nf = 2;
     }
   } else {
-    const int k = (l >> 1) / a.nsub;
-    fkind[nf] = kFInter; fk[nf] = k; ftau[nf++] = dts;
-    if (l & 1) {  // even bonds: both sites' rotations, Y before X
-      fkind[nf] = kFYl; fk[nf] = k; ftau[nf++] = dts;
-      fkind[nf] = kFYr; fk[nf] = k; ftau[nf++] = dts;
-      fkind[nf] = kFXl; fk[nf] = k; ftau[nf++] = dts;
-      fkind[nf] = kFXr; fk[nf] = k; ftau[nf++] = dts;
-    } else if ((N & 1) && b == N - 2) {  // the last site of an odd chain
-      fkind[nf] = kFYr; fk[nf] = k; ftau[nf++] = dts;
-      fkind[nf] = kFXr; fk[nf] = k; ftau[nf++] = dts;
-    }
+    k0 = k1 = (l >> 1) / a.nsub;
+    tau = dts;
+    kind0 = kFInter;
+    // even bonds: both sites' rotations, Y before X; else the last site of an odd chain
+    nf = (l & 1) ? 5 : ((N & 1) && b == N - 2) ? 3 : 1;
   }
+  auto fkind = [&](int f) {
+    if (a.order == 2 || f == 0) return kind0;
+    if (nf == 3) return f == 1 ? kFYr : kFXr;
+    return f == 1 ? kFYl : f == 2 ? kFYr : f == 3 ? kFXl : kFXr;
+  };
+  auto fbin = [&](int f) { return f == 0 ? k0 : k1; };
 
   const double* Jb = a.J + ((size_t)s * nb + b) * a.terms;
   const double jz = Jb[a.terms - 1];
@@ -201,206 +244,224 @@ __global__ void layer_gate_kernel(LayerGateArgs a) {
   const double jy = (a.terms == 3) ? Jb[1] : 0.0;
   const double wl = (b == 0) ? 1.0 : 0.5;
   const double wr = (b + 1 == N - 1) ? 1.0 : 0.5;
+  const unsigned char* mk = a.mask;
 
-  // eigendecomposition and exponential of every factor
-  double2 Vf[kMaxFactors][16], Gf[kMaxFactors][16];
-  double lamf[kMaxFactors][4];
-  for (int f = 0; f < nf; ++f) {
-    const int k = fk[f];
+  // eigendecomposition, exponential and divided differences, two factors at a time
+  const int nfw = (int)__reduce_max_sync(0xffffffffu, (unsigned)nf);
+#pragma unroll 1
+  for (int f0 = 0; f0 < nfw; f0 += 2) {
+    const bool mine = f0 + half < nf;
+    const int f = mine ? f0 + half : 0;
+    const int kind = fkind(f), k = fbin(f);
     const double* uk = a.u + (size_t)k * a.C * N;
-    const unsigned char* mk = a.mask;
-    const double xl = uk[b] * mk[b];
-    const double yl = uk[N + b] * mk[N + b];
-    const double xr = uk[b + 1] * mk[b + 1];
-    const double yr = uk[N + b + 1] * mk[N + b + 1];
+    const double xl = uk[b] * mk[b], yl = uk[N + b] * mk[N + b];
+    const double xr = uk[b + 1] * mk[b + 1], yr = uk[N + b + 1] * mk[N + b + 1];
     double c = jz;
     if (a.C == 3) c += uk[2 * N + b] * mk[2 * N + b];
     if (a.gfix) c += a.gfix[(size_t)k * nb + b];
-    double2 h[16];
+    double2 h[4], v[4];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) h[i] = make_double2(0.0, 0.0);
-    if (fkind[f] == kFBond || fkind[f] == kFInter) {
-      h[0].x = c;
-      h[5].x = -c;
-      h[10].x = -c;
-      h[15].x = c;
-      // J^x XX + J^y YY: <00|.|11> = jx - jy, <01|.|10> = jx + jy
-      h[0 * 4 + 3].x += jx - jy;
-      h[3 * 4 + 0].x += jx - jy;
-      h[1 * 4 + 2].x += jx + jy;
-      h[2 * 4 + 1].x += jx + jy;
-      if (fkind[f] == kFBond) {
-        // (x X + y Y) on a site couples |0> <-> |1> with <0|.|1> = x - i y
-        const double2 lz = make_double2(wl * xl, -wl * yl);
-        const double2 rz = make_double2(wr * xr, -wr * yr);
-        for (int q = 0; q < 2; ++q) {
-          h[(0 + q) * 4 + (2 + q)] = lz;
-          h[(2 + q) * 4 + (0 + q)] = cconj(lz);
-          h[(2 * q) * 4 + (2 * q + 1)] = rz;
-          h[(2 * q + 1) * 4 + (2 * q)] = cconj(rz);
-        }
-      }
-    } else {
-      const int code = fkind[f] - kFXl;  // 0 X(x)I, 1 Y(x)I, 2 I(x)X, 3 I(x)Y
-      const double amp = (code == 0) ? xl : (code == 1) ? yl : (code == 2) ? xr : yr;
-      generator4(code, amp, h);
-    }
-    if (!herm_eig4(h, Vf[f], lamf[f])) atomicOr(a.status, kStatusNoConverge);
-    double2 E[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      double sn, cs;
-      sincos(ftau[f] * lamf[f][j], &sn, &cs);
-      E[j] = make_double2(cs, -sn);
-    }
-#pragma unroll
-    for (int rr = 0; rr < 4; ++rr)
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        double2 g = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) cfma(g, Vf[f][rr * 4 + j], cmulc(E[j], Vf[f][cc * 4 + j]));
-        Gf[f][rr * 4 + cc] = g;
-      }
-  }
-
-  // walk the factors backwards: Lt = product of the factors after f
-  LayerGate& out = a.out[idx];
-  double2 Lt[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) Lt[i] = make_double2((i % 5 == 0) ? 1.0 : 0.0, 0.0);
-  int nq = 0;
-  for (int f = nf - 1; f >= 0; --f) {
-    const int k = fk[f];
-    // the controls of this factor: (generator code, weight, c, site)
-    int pc[5], pcc[5], psite[5];
-    double pw[5];
-    int np = 0;
-    const unsigned char* mk = a.mask;
-    if (fkind[f] == kFBond) {
-      if (mk[b]) { pc[np] = 0; pw[np] = wl; pcc[np] = 0; psite[np++] = b; }
-      if (mk[N + b]) { pc[np] = 1; pw[np] = wl; pcc[np] = 1; psite[np++] = b; }
-      if (mk[b + 1]) { pc[np] = 2; pw[np] = wr; pcc[np] = 0; psite[np++] = b + 1; }
-      if (mk[N + b + 1]) { pc[np] = 3; pw[np] = wr; pcc[np] = 1; psite[np++] = b + 1; }
-    }
-    if ((fkind[f] == kFBond || fkind[f] == kFInter) && a.C == 3 && mk[2 * N + b]) {
-      pc[np] = 4; pw[np] = 1.0; pcc[np] = 2; psite[np++] = b;
-    }
-    if (fkind[f] >= kFXl) {
-      const int code = fkind[f] - kFXl;
-      const int cidx = code & 1, site = b + (code >> 1);
-      if (mk[cidx * N + site]) { pc[np] = code; pw[np] = 1.0; pcc[np] = cidx; psite[np++] = site; }
-    }
-    // Gam_ij e^{i tau lam_j} = -i tau e^{-i tau (lam_i - lam_j)/2} sinc(tau (lam_i - lam_j)/2):
-    // one sincos per entry, shared by every control of the factor
-    double2 GE[16];
-    {
-      const double tau = ftau[f];
-      const double* lam = lamf[f];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const double x = 0.5 * tau * (lam[i] - lam[j]);
-          double sn, cs;
-          sincos(x, &sn, &cs);
-          const double sinc = (fabs(x) < 1e-8) ? 1.0 - x * x / 6.0 : sn / x;
-          // -i tau sinc (cs - i sn) = tau sinc (-sn - i cs)
-          GE[i * 4 + j] = make_double2(-tau * sinc * sn, -tau * sinc * cs);
-        }
-    }
-    for (int q = 0; q < np; ++q) {
-      // Q_f = V (Gam o (V^dag P V)) e^{i tau Lam} V^dag  (= dG_f G_f^dag)
-      double2 P[16], T1[16], T2[16];
-      generator4(pc[q], pw[q], P);
-      const double2* V = Vf[f];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)       // T1 = P V
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) cfma(acc, P[i * 4 + m], V[m * 4 + j]);
-          T1[i * 4 + j] = acc;
-        }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)       // T2 = (Gam o (V^dag T1)) e^{i tau Lam}
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) cfmac(acc, V[m * 4 + i], T1[m * 4 + j]);
-          T2[i * 4 + j] = cmul(GE[i * 4 + j], acc);
-        }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)       // T1 = T2 V^dag
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) cfma(acc, T2[i * 4 + m], cconj(V[j * 4 + m]));
-          T1[i * 4 + j] = acc;
-        }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)       // T2 = V T1  (= dG_f G_f^dag)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) cfma(acc, V[i * 4 + m], T1[m * 4 + j]);
-          T2[i * 4 + j] = acc;
-        }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)       // T1 = T2 Lt^dag
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) cfma(acc, T2[i * 4 + m], cconj(Lt[j * 4 + m]));
-          T1[i * 4 + j] = acc;
-        }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)       // T2 = Lt T1
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) cfma(acc, Lt[i * 4 + m], T1[m * 4 + j]);
-          T2[i * 4 + j] = acc;
-        }
-      const int slot = (k * a.C + pcc[q]) * N + psite[q];
-      int at = -1;
-      for (int e = 0; e < nq; ++e)
-        if (out.slot[e] == slot) at = e;
-      if (at < 0 && nq < kMaxLayerParams) {
-        at = nq++;
-        out.slot[at] = slot;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) out.Q[at][i] = T2[i];
-      } else if (at >= 0) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) out.Q[at][i] = make_double2(out.Q[at][i].x + T2[i].x, out.Q[at][i].y + T2[i].y);
-      } else {
-        atomicOr(a.status, kStatusBadDims);   // cannot happen: at most 10 distinct controls
-      }
-    }
-    // Lt <- Lt G_f
-    double2 T[16];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int j = 0; j < 4; ++j) h[j] = make_double2(0.0, 0.0);
+    if (kind == kFBond || kind == kFInter) {
+      // J^x XX + J^y YY: <00|.|11> = jx - jy, <01|.|10> = jx + jy; (x X + y Y) on
+      // a site couples |0> <-> |1> with <0|.|1> = x - i y
+      const bool bond = kind == kFBond;
+      const double2 lz = make_double2(bond ? wl * xl : 0.0, bond ? ((r & 2) ? wl * yl : -wl * yl) : 0.0);
+      const double2 rz = make_double2(bond ? wr * xr : 0.0, bond ? ((r & 1) ? wr * yr : -wr * yr) : 0.0);
+      const double dg = (r == 0 || r == 3) ? c : -c, cr = (r == 0 || r == 3) ? jx - jy : jx + jy;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        double2 acc = make_double2(0.0, 0.0);
+        if (j == r) h[j] = make_double2(dg, 0.0);
+        if (j == (r ^ 3)) h[j] = make_double2(cr, 0.0);
+        if (j == (r ^ 2)) h[j] = lz;
+        if (j == (r ^ 1)) h[j] = rz;
+      }
+    } else {
+      const int code = kind - kFXl;  // 0 X(x)I, 1 Y(x)I, 2 I(x)X, 3 I(x)Y
+      int col;
+      double2 val;
+      generator_row(code, (code == 0) ? xl : (code == 1) ? yl : (code == 2) ? xr : yr, r, col, val);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) cfma(acc, Lt[i * 4 + m], Gf[f][m * 4 + j]);
-        T[i * 4 + j] = acc;
+      for (int j = 0; j < 4; ++j)
+        if (j == col) h[j] = val;
+    }
+    const bool ok = herm_eig4_rows(h, v, r);
+    if (live && mine && r == 0 && !ok) atomicOr(a.status, kStatusNoConverge);
+    double lam = h[0].x;
+#pragma unroll
+    for (int j = 1; j < 4; ++j)
+      if (j == r) lam = h[j].x;
+    // the exponential E_j = e^{-i tau lam_j}, and e_j = e^{-i tau lam_j / 2}, whose
+    // products e_i conj(e_j) are the half differences
+    double sn, cs;
+    sincos(tau * lam, &sn, &cs);
+    const double2 E = make_double2(cs, -sn);
+    sincos(0.5 * tau * lam, &sn, &cs);
+    const double2 eh = make_double2(cs, -sn);
+    double2 ge[4], vE[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      // Gam_rj e^{i tau lam_j} = -i tau e^{-i x} sinc(x), x = tau (lam_r - lam_j) / 2
+      const double2 ej = shfl4(eh, j);
+      const double x = 0.5 * tau * (lam - __shfl_sync(0xffffffffu, lam, j, 4));
+      const double2 ex = cmulc(eh, ej);   // e^{-i x}
+      const double sc = tau * sinc_of(x, -ex.y);
+      ge[j] = make_double2(sc * ex.y, -sc * ex.x);
+      vE[j] = cmul(v[j], shfl4(E, j));
+    }
+    if (mine) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        S.V[f][r * 4 + j] = v[j];
+        S.GE[f][r * 4 + j] = ge[j];
+      }
+    }
+    __syncwarp();
+    if (mine) {
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {   // G = V E V^dagger
+        double2 g = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cfmac(g, S.V[f][cc * 4 + j], vE[j]);
+        S.G[f][r * 4 + cc] = g;
+      }
+    }
+    __syncwarp();
+  }
+
+  // walk the factors backwards: Lt = product of the factors after f, row r in lt
+  LayerGate& out = a.out[idx];
+  double2 lt[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    lt[j] = make_double2(j == r ? 1.0 : 0.0, 0.0);
+    if (half == 0) S.Lt[r * 4 + j] = lt[j];
+  }
+  __syncwarp();
+  int nq = 0;
+#pragma unroll 1
+  for (int f1 = nfw - 1; f1 >= 0; --f1) {
+    const bool on = f1 < nf;
+    const int f = on ? f1 : 0;
+    const int kind = fkind(f), k = fbin(f);
+    const bool last = f == nf - 1;   // Lt = 1
+    // the controls of this factor, as bits of their generator codes
+    unsigned ctl = 0;
+    if (on) {
+      if (kind == kFBond)
+        ctl = (mk[b] ? 1u : 0u) | (mk[N + b] ? 2u : 0u) | (mk[b + 1] ? 4u : 0u) | (mk[N + b + 1] ? 8u : 0u);
+      if ((kind == kFBond || kind == kFInter) && a.C == 3 && mk[2 * N + b]) ctl |= 16u;
+      if (kind >= kFXl) {
+        const int code = kind - kFXl;
+        if (mk[(code & 1) * N + b + (code >> 1)]) ctl |= 1u << code;
+      }
+    }
+    const int np = __popc(ctl);
+    // both half steps of one bin: their matrices add up in the same records
+    const bool again = on && !last && a.order == 2 && k0 == k1;
+    const int base = again ? 0 : nq;
+    const int npw = (int)__reduce_max_sync(0xffffffffu, (unsigned)np);
+    const bool any_lt = __any_sync(0xffffffffu, on && !last);
+#pragma unroll 1
+    for (int q0 = 0; q0 < npw; q0 += 2) {
+      const int q = q0 + half;
+      const bool mine = q < np;
+      unsigned rest = ctl;
+#pragma unroll 1
+      for (int i = 0; i < q && mine; ++i) rest &= rest - 1;
+      const int code = mine ? __ffs(rest) - 1 : 0;
+      const double w = kind != kFBond || code == 4 ? 1.0 : code < 2 ? wl : wr;
+      // row r of T = (Gam o (V^dag P V)) e^{i tau Lam}, then of T V^dag
+      double2 t[4], u[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) t[j] = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {   // (V^dag P V)[r][j] = sum_m conj(V[m][r]) P[m][col] V[col][j]
+        int col;
+        double2 val;
+        generator_row(code, w, m, col, val);
+        const double2 x = cmulc(val, S.V[f][m * 4 + r]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cfma(t[j], x, S.V[f][col * 4 + j]);
       }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) Lt[i] = T[i];
-  }
+      for (int j = 0; j < 4; ++j) t[j] = cmul(S.GE[f][r * 4 + j], t[j]);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) out.G[i] = Lt[i];
-  out.nq = nq;
+      for (int j = 0; j < 4; ++j) {
+        u[j] = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) cfmac(u[j], S.V[f][j * 4 + m], t[m]);
+        S.T[half][r * 4 + j] = u[j];
+      }
+      __syncwarp();
+      // Q_f = V (T V^dag)  (= dG_f G_f^dag)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        t[j] = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) cfma(t[j], S.V[f][r * 4 + m], S.T[half][m * 4 + j]);
+      }
+      __syncwarp();
+      if (any_lt) {   // L Q_f L^dag
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          u[j] = make_double2(0.0, 0.0);
+#pragma unroll
+          for (int m = 0; m < 4; ++m) cfmac(u[j], S.Lt[j * 4 + m], t[m]);
+          S.T[half][r * 4 + j] = u[j];
+        }
+        __syncwarp();
+        if (!last) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            t[j] = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) cfma(t[j], lt[m], S.T[half][m * 4 + j]);
+          }
+        }
+        __syncwarp();
+      }
+      if (live && mine) {
+        const int at = base + q;   // at most 10 distinct controls: kMaxLayerParams
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (again) {
+            const double2 o = out.Q[at][r * 4 + j];
+            t[j].x += o.x;
+            t[j].y += o.y;
+          }
+          out.Q[at][r * 4 + j] = t[j];
+        }
+        if (r == 0) {
+          const int cidx = code == 4 ? 2 : (code & 1), site = (code == 2 || code == 3) ? b + 1 : b;
+          out.slot[at] = (k * a.C + cidx) * N + site;
+        }
+      }
+    }
+    if (on && !again) nq += np;
+    // Lt <- Lt G_f
+    double2 x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      x[j] = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) cfma(x[j], lt[m], S.G[f][m * 4 + j]);
+    }
+    __syncwarp();
+    if (on) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        lt[j] = x[j];
+        if (half == 0) S.Lt[r * 4 + j] = x[j];
+      }
+    }
+    __syncwarp();
+  }
+  if (live && half == 0) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out.G[r * 4 + j] = lt[j];
+    if (r == 0) out.nq = nq;
+  }
 }
 
 __device__ __forceinline__ unsigned long long splitmix64(unsigned long long seed, unsigned long long i) {
@@ -460,8 +521,8 @@ extern "C" cudaError_t tnrc_launch_layer_gates(int N, int K, int C, int M, int t
                                                cudaStream_t st) {
   tnrc::LayerGateArgs a{N, K, C, M, terms, order, nsub, L, R, first_parity, dt, u, mask, gfix, J, layer_off, out,
                         status};
-  const long long total = (long long)M * R;
-  const int threads = 64;
+  const long long total = (long long)M * R * tnrc::kRecLanes;
+  const int threads = tnrc::kGateThreads;
   const long long blocks = (total + threads - 1) / threads;
   (void)cudaGetLastError();  // report only this launch below
   tnrc::layer_gate_kernel<<<(unsigned)blocks, threads, 0, st>>>(a);
