@@ -291,22 +291,17 @@ __global__ void __launch_bounds__(kGateThreads) layer_gate_kernel(LayerGateArgs 
 #pragma unroll
     for (int j = 1; j < 4; ++j)
       if (j == r) lam = h[j].x;
-    // the exponential E_j = e^{-i tau lam_j}, and e_j = e^{-i tau lam_j / 2}, whose
-    // products e_i conj(e_j) are the half differences
     double sn, cs;
     sincos(tau * lam, &sn, &cs);
-    const double2 E = make_double2(cs, -sn);
-    sincos(0.5 * tau * lam, &sn, &cs);
-    const double2 eh = make_double2(cs, -sn);
+    const double2 E = make_double2(cs, -sn);   // e^{-i tau lam_r}
     double2 ge[4], vE[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       // Gam_rj e^{i tau lam_j} = -i tau e^{-i x} sinc(x), x = tau (lam_r - lam_j) / 2
-      const double2 ej = shfl4(eh, j);
       const double x = 0.5 * tau * (lam - __shfl_sync(0xffffffffu, lam, j, 4));
-      const double2 ex = cmulc(eh, ej);   // e^{-i x}
-      const double sc = tau * sinc_of(x, -ex.y);
-      ge[j] = make_double2(sc * ex.y, -sc * ex.x);
+      sincos(x, &sn, &cs);
+      const double sc = tau * sinc_of(x, sn);
+      ge[j] = make_double2(-sc * sn, -sc * cs);
       vE[j] = cmul(v[j], shfl4(E, j));
     }
     if (mine) {

@@ -79,7 +79,7 @@ __device__ int plain_share(const TrajParams& p, const int* D, int j, int& nb, in
   }
   __syncwarp();
   nb = left;
-  e = 2 * (j - nw);
+  e = group_size(p) * (j - nw);
   return wide;
 }
 

@@ -511,9 +511,13 @@ __device__ __forceinline__ void fx_circle(int m1, int r, int q, int& i, int& j) 
   }
 }
 
+// |cos|^2 between two columns below which they count as orthogonal: 4 units of
+// FP64 rounding (the integer inner products resolve a quarter of one)
+constexpr float kFxTol2 = 1e-30f;
+
 // Pair (i, j) by its group of lanes; called by whole warps.
 template <bool SH>
-__device__ __forceinline__ void fx_pair(const FxMem<SH>& X, int ldx, int n, int i, int j, bool on, float tol2, int* ex,
+__device__ __forceinline__ void fx_pair(const FxMem<SH>& X, int ldx, int n, int i, int j, bool on, int* ex,
                                         int lig, int lg, int lgm, int& rotated, int& large) {
   const int oa = i * ldx, ob = j * ldx, nr = on ? n : 0;
   FxAcc sa{0, 0}, sb{0, 0}, re{0, 0}, im{0, 0};
@@ -541,7 +545,7 @@ __device__ __forceinline__ void fx_pair(const FxMem<SH>& X, int ldx, int n, int 
   const float af = fx_to_float(aa) * k40, bf = fx_to_float(bb) * k40;
   const float xr = fx_to_float(abr) * k40, xi = fx_to_float(abi) * k40;
   const float ab2 = fmaf(xr, xr, xi * xi), pab = af * bf;
-  if (on && ab2 > tol2 * pab) {
+  if (on && ab2 > kFxTol2 * pab) {
     FxRot R;
     fx_rotation(aa, bb, abr, abi, ej - ei, af, bf, xr, xi, ab2, R);
     rotated = 1;
@@ -581,10 +585,6 @@ __device__ __forceinline__ void fx_pair(const FxMem<SH>& X, int ldx, int n, int 
   }
 }
 
-__device__ __forceinline__ float fx_tol2(int n, int m) {
-  const float tol = 2.0f * (float)(m > n ? m : n) * 2.220446e-16f;
-  return tol * tol;
-}
 
 static __device__ __noinline__ int fx_jacobi(int4* Xp, int ldx, int n, int m, const int* xe, int* ex, int lane, int lw) {
   const FxMem<true> X(Xp);
@@ -605,7 +605,6 @@ static __device__ __noinline__ int fx_jacobi(int4* Xp, int ldx, int n, int m, co
   const int lg = fx_lanes(trivial ? lw : Pe, lw), gi = ll >> lg, lig = ll & ((1 << lg) - 1), groups = lw >> lg;
   const int iters = fx_umax(trivial ? 0 : (Pe + groups - 1) / groups), lgm = fx_umax(lg);
   const int rounds = fx_umax(trivial ? 0 : m1);
-  const float tol2 = fx_tol2(n, m);
   bool active = !trivial;
   int result = trivial ? ((m < 1 || n < 1) ? 0 : 1) : -kMaxSweeps;
   for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
@@ -619,7 +618,7 @@ static __device__ __noinline__ int fx_jacobi(int4* Xp, int ldx, int n, int m, co
         const bool on = active && r < m1 && q < P;
         int i = 0, j = 0;
         if (on) fx_circle(m1, r, q, i, j);
-        fx_pair(X, ldx, n, i, j, on, tol2, ex, lig, lg, lgm, rotated, large);
+        fx_pair(X, ldx, n, i, j, on, ex, lig, lg, lgm, rotated, large);
       }
       __syncwarp();
     }
@@ -648,7 +647,6 @@ __device__ __noinline__ int fx_jacobi_cta(int4* Xp, int ldx, int n, int m, const
   if (m < 1 || n < 1) return 0;
   if (Pe < 1) return 1;
   const int lg = fx_cta_lanes(Pe), gi = ti >> lg, lig = ti & ((1 << lg) - 1), groups = nt >> lg;
-  const float tol2 = fx_tol2(n, m);
   for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
     int rotated = 0, large = 0;
 #pragma unroll 1
@@ -659,7 +657,7 @@ __device__ __noinline__ int fx_jacobi_cta(int4* Xp, int ldx, int n, int m, const
         const bool on = q < P;
         int i = 0, j = 0;
         if (on) fx_circle(m1, r, q, i, j);
-        fx_pair(X, ldx, n, i, j, on, tol2, ex, lig, lg, lg, rotated, large);
+        fx_pair(X, ldx, n, i, j, on, ex, lig, lg, lg, rotated, large);
       }
       __syncthreads();
     }

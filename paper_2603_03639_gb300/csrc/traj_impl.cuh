@@ -177,91 +177,189 @@ __device__ __noinline__ double theta_build(const TrajParams& p, const Lay& Y, un
 }
 
 // Phase 3 of a two-site update of bond b, by one warp, after the SVD left
-// R^dagger V = Z S in T (r columns of length n): rank and truncate, lam_b <-
-// S_k / |S_k|, 1 / sigma of the kept values in bf.qn, ranks in bf.perm.
-// Returns k; inv_kn = 1 / |S_k|.
+// R^dagger V = Z S in X (r columns of length n, real values X 2^ex[j]): rank and
+// truncate, lam_b <- S_k / |S_k|.  Keeps k = max(1, min(chi, #{sigma_j > eps
+// sigma_max})); bf.perm[i] = column of rank i, by decreasing sigma with ties to
+// the smaller index.  nrm[j] (r entries) receives what normalises column j: y =
+// 1 / |X_j| for X_j shifted by the number in bf.piv[j].  Returns k; inv_kn =
+// 1 / |S_k|.  In integers but for the squared values that are ranked and the
+// Schmidt values themselves: with FP64 sums, roots and quotients this took 8,500
+// cycles of a small update's 65,000.
+struct ColNorm {
+  long long n2, y;
+};
 template <int kD>
-__device__ __noinline__ int theta_rank(const TrajParams& p, const Lay& Y, unsigned char* slot, int b, const double2* T, int r,
-                          int sw, bool record, bool count, WarpCtx& w, SvdBufs bf, double& inv_kn) {
+__device__ __noinline__ int theta_rank(const TrajParams& p, const Lay& Y, unsigned char* slot, int b, const int4* X,
+                                       int ldx, const int* ex, ColNorm* nrm, int r, int sw, bool record, bool count,
+                                       WarpCtx& w, SvdBufs bf, double& inv_kn) {
   const int lane = w.lane;
   const int* D = slot_dims(slot);
-  const int Dl = D[b], Dc = D[b + 1], Dr = D[b + 2];
-  const int m = kD * Dl, n = kD * Dr;
-  double* lam = slot_lam(slot, Y.L);
-  double kept2, tot2, gap;
-  int k = warp_rank_truncate(T, n, r, p.chi, p.eps, bf.sig2, bf.perm, lane, kept2, tot2, gap);
+  const int m = kD * D[b], n = kD * D[b + 2];
+  {
+    const int lg = fx_lanes(r, 32), gi = lane >> lg, lig = lane & ((1 << lg) - 1), groups = 32 >> lg;
+#pragma unroll 1
+    for (int c0 = 0; c0 < r; c0 += groups) {
+      const int c = c0 + gi;
+      FxAcc nn{0, 0};
+      if (c < r)
+#pragma unroll 1
+        for (int i = lig; i < n; i += 1 << lg) fx_cabs2(nn, X[c * ldx + i]);
+      const long long N = fx_group_sum(fx_sum2(nn), lg, lg);
+      if (c < r && lig == 0) nrm[c].n2 = N;
+    }
+  }
+  __syncwarp();
+  // sigma_j^2 = n2 2^(56 + 2 e), n2 in [2^54, 2^56), e = ex - shift
+  int emax = -100000;
+  double mx = 0.0;
+#pragma unroll 1
+  for (int j = lane; j < r; j += 32) {
+    long long N = nrm[j].n2;
+    int z = 0;
+    double sq = 0.0;
+    if (N > 0) {
+      z = (55 - (63 - __clzll(N))) >> 1;
+      N = z >= 0 ? N << (2 * z) : N >> (-2 * z);
+      emax = max(emax, ex[j] - z);
+      sq = fx_scale((double)N, 56 + 2 * (ex[j] - z));
+      nrm[j].y = fx_rsqrt(N);
+    } else {
+      nrm[j].y = 0;
+    }
+    nrm[j].n2 = N;
+    bf.piv[j] = z;
+    bf.sig2[j] = sq;
+    mx = fmax(mx, sq);
+  }
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+    const long long v = __shfl_xor_sync(0xffffffffu, __double_as_longlong(mx), o);
+    if (v > __double_as_longlong(mx)) mx = __longlong_as_double(v);
+  }
+  __syncwarp();
+  const double cut2 = p.eps * p.eps * mx;
+  int cnt = 0;
+  long long tot = 0;
+#pragma unroll 1
+  for (int j = lane; j < r; j += 32) {
+    cnt += bf.sig2[j] > cut2 ? 1 : 0;
+    const int d = 2 * (emax - ex[j] + bf.piv[j]);
+    tot += d < 63 ? nrm[j].n2 >> d : 0;
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  int k = cnt < p.chi ? cnt : p.chi;
+  if (k > n) k = n;  // at most n orthogonal columns of length n
+  if (k < 1) k = 1;
+  long long kept = 0;
+#pragma unroll 1
+  for (int j = lane; j < r; j += 32) {
+    const long long vj = __double_as_longlong(bf.sig2[j]);
+    int rk = 0;
+#pragma unroll 1
+    for (int i = 0; i < r; ++i) {
+      const long long vi = __double_as_longlong(bf.sig2[i]);
+      rk += (vi > vj || (vi == vj && i < j)) ? 1 : 0;
+    }
+    if (rk <= k) bf.perm[rk] = j;
+    const int d = 2 * (emax - ex[j] + bf.piv[j]);
+    if (rk < k) kept += d < 63 ? nrm[j].n2 >> d : 0;
+  }
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    kept += __shfl_xor_sync(0xffffffffu, kept, o);
+  }
+  __syncwarp();
+  const double kept2 = fx_scale((double)kept, 56 + 2 * emax);
+  if (lane == 0) {
+    if (sw < 0) atomicOr(p.status, kStatusNoConverge);
+    if (!(kept2 > 0.0)) atomicOr(p.status, kStatusNaN);
+  }
+  // the relative distance between the last kept and the first dropped value,
+  // when the cap chi decided the cut
+  const bool capped = cnt > k && k < r;
   if (k > Y.dcap[b + 1]) {  // cannot happen (k <= min(m, n, chi)); keeps memory in bounds regardless
     k = Y.dcap[b + 1];
     if (lane == 0) atomicOr(p.status, kStatusBadDims);
   }
-  if (lane == 0) {
-    if (sw < 0) atomicOr(p.status, kStatusNoConverge);
-    if (!(tot2 >= 0.0) || !(tot2 < 1e300) || !(kept2 > 0.0)) atomicOr(p.status, kStatusNaN);
-  }
   w.sweeps += (sw < 0) ? -sw : sw;
   w.updates += 1;
   if (record) {
-    w.disc += fmax(0.0, tot2 - kept2) / tot2;   // rounding can make tot2 - kept2 slightly negative
+    w.disc += tot > kept ? (double)(tot - kept) / (double)tot : 0.0;
     if (k > w.maxk) w.maxk = k;
     if (lane == 0) atomicAdd(&p.counters[kCtrHist + k], 1ull);
   }
   if (count) {
-    w.alg += update_flops(m, n, Dc, k);
-    if (gap >= 0.0) {   // the cap chi_max decided this cut
+    w.alg += update_flops(m, n, D[b + 1], k);
+    if (capped) {
       w.capcuts += 1;
+      const double gap = (sqrt(bf.sig2[bf.perm[k - 1]]) - sqrt(bf.sig2[bf.perm[k]])) / sqrt(mx);
       if (lane == 0) atomicMin(&p.counters[kCtrGap], (unsigned long long)__double_as_longlong(gap));
     }
   }
   inv_kn = rsqrt(kept2);
-  // 1 / sigma once per kept value, in qn, which the Jacobi no longer needs
-  double* lamw = lam + (size_t)b * Y.L.chi;
+  double* lamw = slot_lam(slot, Y.L) + (size_t)b * Y.L.chi;
 #pragma unroll 1
   for (int i = lane; i < k; i += 32) {
-    lamw[i] = sqrt(bf.sig2[bf.perm[i]]) * inv_kn;
-    bf.qn[i] = rsqrt(bf.sig2[bf.perm[i]]);
+    const int j = bf.perm[i];
+    const long long s = fx_mul(fx_split(nrm[j].n2), fx_split(nrm[j].y));   // |X_j| 2^shift
+    lamw[i] = fx_scale((double)s, ex[j] - bf.piv[j]) * inv_kn;
   }
   __syncwarp();
   return k;
 }
 
-// Phase 4, by thread ti of nt: B_{b+1} <- Y_k^dag, B_b <- Phi Y_k / |S_k|,
-// with column i of Y_k = T[perm[i] n + .] / sigma_i.
+// Row i of Y_k^dagger, y_i = X_j / |X_j| with j = perm[i], into T (FP64), by
+// thread ti of nt.
+__device__ __forceinline__ void right_vectors(const int4* X, int ldx, const ColNorm* nrm, const SvdBufs& bf, int n, int k,
+                                              double2* T, int ti, int nt) {
+#pragma unroll 1
+  for (int it = ti; it < k * n; it += nt) {
+    const int i = it / n, c = it - i * n, j = bf.perm[i];
+    const int4 z = fx_shift(X[j * ldx + c], bf.piv[j]);
+    const Fx y = fx_split(nrm[j].y);
+    T[it] = make_double2(fx_scale((double)fx_mul(fx_re(z), y), -56), fx_scale((double)fx_mul(fx_im(z), y), -56));
+  }
+}
+
+// Phase 4, by thread ti of nt: B_{b+1} <- Y_k^dag, B_b <- Phi Y_k / |S_k|, with
+// column i of Y_k = T[i n + .].
 template <int kD>
-__device__ __noinline__ void theta_split(const Lay& Y, unsigned char* slot, int b, const double2* T, const double2* Phi, int k,
-                            SvdBufs bf, double inv_kn, int ti, int nt) {
+__device__ __noinline__ void theta_split(const Lay& Y, unsigned char* slot, int b, const double2* T, const double2* Phi,
+                                         int k, double inv_kn, int ti, int nt) {
   const int* D = slot_dims(slot);
   const int m = kD * D[b], n = kD * D[b + 2];
   double2* sites = slot_sites(slot, Y.L);
   double2* A = sites + Y.site_off[b];
   double2* Bt = sites + Y.site_off[b + 1];
-  const double* isig = bf.qn;
 #pragma unroll 1
-  for (int it = ti; it < k * n; it += nt) {
-    const int i = it / n, c = it - i * n;
-    Bt[it] = cscale(cconj(T[(size_t)bf.perm[i] * n + c]), isig[i]);
-  }
+  for (int it = ti; it < k * n; it += nt) Bt[it] = cconj(T[it]);
 #pragma unroll 1
   for (int it = ti; it < m * k; it += nt) {
     const int row = it / k, i = it - row * k;
     const double2* ph = Phi + (size_t)row * n;
-    const double2* z = T + (size_t)bf.perm[i] * n;
+    const double2* z = T + (size_t)i * n;
     double2 acc = make_double2(0.0, 0.0);
 #pragma unroll 1
     for (int c = 0; c < n; ++c) cfma(acc, ph[c], z[c]);
-    A[it] = cscale(acc, isig[i] * inv_kn);
+    A[it] = cscale(acc, inv_kn);
   }
 }
 
 // Phases 3 and 4 by one warp.
 template <int kD>
-__device__ void theta_finish(const TrajParams& p, const Lay& Y, unsigned char* slot, int b, const double2* T,
-                             const double2* Phi, int r, int sw, bool record, bool count, WarpCtx& w, SvdBufs bf) {
+__device__ __noinline__ void theta_finish(const TrajParams& p, const Lay& Y, unsigned char* slot, int b, const int4* X,
+                                          int ldx, const int* ex, ColNorm* nrm, double2* T, const double2* Phi, int r,
+                                          int sw, bool record, bool count, WarpCtx& w, SvdBufs bf) {
   TNRC_TIC(t_r);
   double inv_kn;
-  const int k = theta_rank<kD>(p, Y, slot, b, T, r, sw, record, count, w, bf, inv_kn);
+  const int k = theta_rank<kD>(p, Y, slot, b, X, ldx, ex, nrm, r, sw, record, count, w, bf, inv_kn);
   TNRC_TOC(w, 2, t_r);
   TNRC_TIC(t_w);
-  theta_split<kD>(Y, slot, b, T, Phi, k, bf, inv_kn, w.lane, 32);
+  right_vectors(X, ldx, nrm, bf, kD * slot_dims(slot)[b + 2], k, T, w.lane, 32);
+  __syncwarp();
+  theta_split<kD>(Y, slot, b, T, Phi, k, inv_kn, w.lane, 32);
   __syncwarp();
   if (w.lane == 0) slot_dims(slot)[b + 1] = k;
   __syncwarp();
@@ -311,10 +409,8 @@ __device__ __noinline__ void two_site_update(const TrajParams& p, const Lay& Y, 
   TNRC_TIC(t_s);
   const int sw = fx_jacobi(X, ldx, n, r, w.perm, ex, lane, 32);
   TNRC_TOC(w, 8, t_s);
-#pragma unroll 1
-  for (int e = lane; e < r * n; e += 32) T[e] = fx_to_double2(X[(e / n) * ldx + e % n], ex[e / n]);
-  __syncwarp();
-  theta_finish<kD>(p, Y, slot, b, T, Phi, r, sw, record, count, w, SvdBufs{w.sig2, w.qn, w.perm, w.piv});
+  theta_finish<kD>(p, Y, slot, b, X, ldx, ex, reinterpret_cast<ColNorm*>(X + (m < n ? m : n) * ldx), T, Phi, r, sw,
+                   record, count, w, SvdBufs{w.sig2, w.qn, w.perm, w.piv});
 }
 
 // Where a wide update keeps theta, Phi and R^dagger: side by side in the
@@ -376,14 +472,12 @@ __device__ __noinline__ void wide_update_cta(const TrajParams& p, const Lay& Y, 
   const int sw = h.shared ? fx_jacobi_cta<true>(X, ldx, n, r, w.cta_perm, ex)
                           : fx_jacobi_cta<false>(X, ldx, n, r, w.cta_perm, ex);
   TNRC_TOC(w, 8, t_s);
-#pragma unroll 1
-  for (int e = ti; e < r * n; e += nt) h.T[e] = fx_to_double2(X[(e / n) * ldx + e % n], ex[e / n]);
-  __syncthreads();
   TNRC_TIC(t_r);
+  ColNorm* nrm = reinterpret_cast<ColNorm*>(Pw);
   const SvdBufs bf{w.cta_sig2, w.cta_qn, w.cta_perm, w.cta_piv};
   if (warp == 0) {
     double inv_kn;
-    const int k = theta_rank<kD>(p, Y, slot, b, h.T, r, sw, record, count, w, bf, inv_kn);
+    const int k = theta_rank<kD>(p, Y, slot, b, X, ldx, ex, nrm, r, sw, record, count, w, bf, inv_kn);
     if (w.lane == 0) {
       ws->k = k;
       ws->part[0] = inv_kn;
@@ -393,7 +487,9 @@ __device__ __noinline__ void wide_update_cta(const TrajParams& p, const Lay& Y, 
   TNRC_TOC(w, 2, t_r);
   TNRC_TIC(t_w);
   const int k = ws->k;
-  theta_split<kD>(Y, slot, b, h.T, h.Phi, k, bf, ws->part[0], ti, nt);
+  right_vectors(X, ldx, nrm, bf, n, k, h.T, ti, nt);
+  __syncthreads();
+  theta_split<kD>(Y, slot, b, h.T, h.Phi, k, ws->part[0], ti, nt);
   __syncthreads();
   if (ti == 0) slot_dims(slot)[b + 1] = k;
   __syncthreads();
@@ -404,6 +500,13 @@ __device__ __noinline__ void wide_update_cta(const TrajParams& p, const Lay& Y, 
 #define TNRC_PAIR_SIDE 64
 #endif
 constexpr int kPairSide = TNRC_PAIR_SIDE;
+// Bonds a warp takes at a time.  Two, with small ones as a pair, where a layer
+// has more bonds than an SM's eight warps twice over; one below that, where
+// pairs would leave warps without a bond (8 qubits, 4 bonds a layer: 5.9 ms
+// two at a time).  By the layer's bonds only, so that results do not depend on
+// the launch.
+__device__ __forceinline__ int group_size(const TrajParams& p) { return p.N - 1 >= 32 ? 2 : 1; }
+
 // Whether bonds b1 and b2 of one layer are updated as a pair: pairing is on
 // for the context (the matrix shape the autotuner picks), both thetas and
 // both Phis fit the warp's shared slab side by side, and every side is at
@@ -478,13 +581,10 @@ __device__ __noinline__ void two_site_update_pair(const TrajParams& p, const Lay
   const int swh = fx_jacobi(Xh, ldh, nh, hi ? r2 : r1, bf.perm, hi ? ex2 : ex1, lane, 16);
   const int sw1 = __shfl_sync(0xffffffffu, swh, 0), sw2 = __shfl_sync(0xffffffffu, swh, 16);
   TNRC_TOC(w, 8, t_s);
-#pragma unroll 1
-  for (int e = lane; e < r1 * n1; e += 32) T1[e] = fx_to_double2(X1[(e / n1) * ld1 + e % n1], ex1[e / n1]);
-#pragma unroll 1
-  for (int e = lane; e < r2 * n2; e += 32) T2[e] = fx_to_double2(X2[(e / n2) * ld2 + e % n2], ex2[e / n2]);
-  __syncwarp();
-  theta_finish<kD>(p, Y, slot, b1, T1, Phi1, r1, sw1, record, count, w, bf1);
-  theta_finish<kD>(p, Y, slot, b2, T2, Phi2, r2, sw2, record, count, w, bf2);
+  theta_finish<kD>(p, Y, slot, b1, X1, ld1, ex1, reinterpret_cast<ColNorm*>(X1 + (m1 < n1 ? m1 : n1) * ld1), T1, Phi1, r1,
+                   sw1, record, count, w, bf1);
+  theta_finish<kD>(p, Y, slot, b2, X2, ld2, ex2, reinterpret_cast<ColNorm*>(X2 + (m2 < n2 ? m2 : n2) * ld2), T2, Phi2, r2,
+                   sw2, record, count, w, bf2);
 }
 
 // ---------------------------------------------------------------------------
@@ -510,43 +610,53 @@ __device__ __forceinline__ StateView packed_view(const unsigned char* rec, int N
   return StateView{D, D + N + 1, reinterpret_cast<const double2*>(rec + packed_header(N))};
 }
 
-// Bytes of the packed record of a slot (same value in every thread).
+// CTA-wide: write the packed record of `slot` to `rec`, unless it takes more than
+// `room` bytes; returns its size (the same in every thread).  Every warp scans
+// the site sizes, then copies every warps-th site: site after site by the whole
+// CTA, with each size read from memory in turn, was a tenth of a small
+// evaluation.
 template <int kD>
-__device__ __forceinline__ size_t packed_bytes(const int* D, int N) {
-  size_t e = 0;
-#pragma unroll 1
-  for (int i = 0; i < N; ++i) e += (size_t)D[i] * kD * D[i + 1];
-  return packed_header(N) + e * 16;
-}
-
-// CTA-wide: write the packed record of `slot` to `rec`.
-template <int kD>
-__device__ __noinline__ void pack_state(const TrajParams& p, const Lay& Y, const unsigned char* slot, unsigned char* rec) {
-  const int N = p.N;
+__device__ __noinline__ size_t pack_state(const TrajParams& p, const Lay& Y, const unsigned char* slot,
+                                          unsigned char* rec, size_t room) {
+  const int N = p.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int* D = slot_dims(slot);
   int* hd = reinterpret_cast<int*>(rec);
   double2* out = reinterpret_cast<double2*>(rec + packed_header(N));
   const double2* src = slot_sites(slot, Y.L);
-  if (threadIdx.x == 0) {
-    int o = 0;
+  int total = 0;
 #pragma unroll 1
-    for (int i = 0; i <= N; ++i) hd[i] = D[i];
+  for (int i = lane; i < N; i += 32) total += D[i] * kD * D[i + 1];
+  total = __reduce_add_sync(0xffffffffu, total);
+  const size_t need = packed_header(N) + (size_t)total * 16;
+  if (need > room) return need;
+  int o = 0;
 #pragma unroll 1
-    for (int i = 0; i < N; ++i) {
-      hd[N + 1 + i] = o;
-      o += D[i] * kD * D[i + 1];
+  for (int i0 = 0; i0 < N; i0 += 32) {
+    const int i = i0 + lane;
+    const int cnt = i < N ? D[i] * kD * D[i + 1] : 0, from = i < N ? Y.site_off[i] : 0;
+    int sum = cnt;
+#pragma unroll 1
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, sum, d);
+      if (lane >= d) sum += v;
     }
-  }
-  size_t o = 0;
+    const int at = o + sum - cnt;
+    if (warp == 0 && i < N) {
+      hd[i] = D[i];
+      hd[N + 1 + i] = at;
+    }
 #pragma unroll 1
-  for (int i = 0; i < N; ++i) {
-    const int cnt = D[i] * kD * D[i + 1];
-    const double2* a = src + Y.site_off[i];
+    for (int u = warp; u < 32 && i0 + u < N; u += nw) {
+      const int c = __shfl_sync(0xffffffffu, cnt, u), f = __shfl_sync(0xffffffffu, from, u),
+                t = __shfl_sync(0xffffffffu, at, u);
 #pragma unroll 1
-    for (int e = threadIdx.x; e < cnt; e += blockDim.x) out[o + e] = a[e];
-    o += cnt;
+      for (int e = lane; e < c; e += 32) out[t + e] = src[f + e];
+    }
+    o += __shfl_sync(0xffffffffu, sum, 31);
   }
+  if (threadIdx.x == 0) hd[N] = D[N];
   __syncthreads();
+  return need;
 }
 
 // ---------------------------------------------------------------------------
@@ -953,7 +1063,7 @@ template <int kD>
 __device__ __noinline__ void forward_group(const TrajParams& p, const Lay& Y, unsigned char* slot, int s, int l, int e, int nb,
                               bool adjoint, bool record, bool count, WarpCtx& w) {
   const int b1 = w.order[e];
-  const int b2 = (e + 1 < nb) ? w.order[e + 1] : -1;
+  const int b2 = (group_size(p) == 2 && e + 1 < nb) ? w.order[e + 1] : -1;
   if (b2 >= 0 && pair_fits<kD>(p, slot_dims(slot), b1, b2)) {
     two_site_update_pair<kD>(p, Y, slot, b1, layer_rec(p, s, l, b1).G, b2, layer_rec(p, s, l, b2).G, adjoint,
                              record, count, w);
@@ -1008,9 +1118,9 @@ __device__ void apply_layer(const TrajParams& p, const Lay& Y, unsigned char* sl
     nb = wide_bonds<kD>(p, slot_dims(slot), nb, w, [&](int b) {
       wide_update_cta<kD>(p, Y, slot, b, layer_rec(p, s, l, b).G, adjoint, record, count, w);
     });
-  for (;;) {   // two bonds at a time
+  for (;;) {
     int e = 0;
-    if (lane == 0) e = atomicAdd(w.next, 2);
+    if (lane == 0) e = atomicAdd(w.next, group_size(p));
     e = __shfl_sync(0xffffffffu, e, 0);
     if (e >= nb) break;
     forward_group<kD>(p, Y, slot, s, l, e, nb, adjoint, record, count, w);
@@ -1028,7 +1138,7 @@ __device__ __noinline__ void costate_group(const TrajParams& p, const Lay& Y, un
                               int l, int e, int nb, double2 wO, double* gsp_row, WarpCtx& w) {
   const int* Dc = slot_dims(cslot);
   const int b1 = w.order[e];
-  const int b2 = (e + 1 < nb) ? w.order[e + 1] : -1;
+  const int b2 = (group_size(p) == 2 && e + 1 < nb) ? w.order[e + 1] : -1;
   if (b2 >= 0 && pair_fits<kD>(p, Dc, b1, b2)) {
     double2* th1 = pair_theta<kD>(p, Dc, b1, 0, w);
     double2* th2 = pair_theta<kD>(p, Dc, b1, 1, w);
@@ -1080,9 +1190,9 @@ __device__ void costate_layer(const TrajParams& p, const Lay& Y, unsigned char* 
       __syncthreads();
       wide_update_cta<kD>(p, Y, cslot, b, layer_rec(p, s, l, b).G, true, false, true, w, th);
     });
-  for (;;) {   // two bonds at a time
+  for (;;) {
     int e = 0;
-    if (lane == 0) e = atomicAdd(w.next, 2);
+    if (lane == 0) e = atomicAdd(w.next, group_size(p));
     e = __shfl_sync(0xffffffffu, e, 0);
     if (e >= nb) break;
     costate_group<kD>(p, Y, cslot, av, s, l, e, nb, wO, gsp_row, w);
@@ -1125,11 +1235,10 @@ __device__ __noinline__ int run_trajectory(const TrajParams& p, bool packed, uns
     apply_layer<kD>(p, Y, a_slot, s, l, false, true, true, w, warp);
     if (p.want_grad) {
       if (packed) {
-        const size_t need = packed_bytes<kD>(slot_dims(a_slot), p.N);
-        if (pos + need > hbytes) return 1;
         TNRC_TIC(t_h);
-        pack_state<kD>(p, Y, a_slot, harena + pos);
+        const size_t room = pos < hbytes ? hbytes - pos : 0, need = pack_state<kD>(p, Y, a_slot, harena + pos, room);
         TNRC_TOC(w, 6, t_h);
+        if (need > room) return 1;
         if (threadIdx.x == 0) hpos[l] = (long long)pos;
         pos += (need + 255) / 256 * 256;
       } else if (q == Y.nseg - 1) {
