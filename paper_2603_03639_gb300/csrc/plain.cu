@@ -118,14 +118,11 @@ template <int kD>
 __global__ void __launch_bounds__(64) plain_envs_kernel(TrajParams p, const unsigned char* cslot,
                                                         const unsigned char* aslot) {
   __shared__ int s_order[1], s_next;
+  __shared__ WideShared s_wide;
   WarpCtx w;
   const int warp = threadIdx.x >> 5;
-  plain_warp(p, w, warp, s_order, &s_next, warp);
-  const size_t cc = (size_t)p.chi * p.chi;
-  if (threadIdx.x == 0) {
-    p.env_scratch[0] = make_double2(1.0, 0.0);
-    p.env_scratch[(size_t)(2 * p.N + 1) * cc] = make_double2(1.0, 0.0);
-  }
+  plain_warp(p, w, warp, s_order, &s_next, warp, &s_wide);
+  layer_to_fx<kD>(p, p.full, cslot, slot_view(aslot, p.full), w);
   __syncthreads();
   layer_envs<kD>(p, p.full, cslot, slot_view(aslot, p.full), w, warp);
 }
@@ -150,7 +147,7 @@ __global__ void __launch_bounds__(32) plain_bwd_kernel(TrajParams p, unsigned ch
     double2* th = wide_home<kD>(p, kD * D[wide], kD * D[wide + 2], w).T;
     bond_gradient<kD>(p, p.full, cslot, slot_view(aslot, p.full), s, l, wide, p.O[t], row, w, th, true);
     __syncthreads();
-    wide_update_cta<kD>(p, p.full, cslot, wide, layer_rec(p, s, l, wide).G, true, false, true, w, th);
+    wide_update_cta<kD>(p, p.full, cslot, wide, layer_rec(p, s, l, wide).G, true, false, true, w, true);
   } else if (e < nb) {
     costate_group<kD>(p, p.full, cslot, slot_view(aslot, p.full), s, l, e, nb, p.O[t], row, w);
   }

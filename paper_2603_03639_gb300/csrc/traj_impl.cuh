@@ -62,6 +62,7 @@ struct WideShared {
   double part[kWarps];
   FxQrShared qr;
   long long total;   // cost of the current layer
+  int ring[6];       // largest entries of the environment steps
   int k;
 };
 
@@ -104,74 +105,60 @@ struct SvdBufs {
 };
 
 // Phase 1 of a two-site update of bond b: Phi = G (B_b B_{b+1}) and theta =
-// lam_{b-1} Phi, both row-major: row (al s1), column (s2 ga).  With `pre` the
-// product B_b B_{b+1} is given ([Dl][kD^2][Dr], the layout of theta itself,
-// so pre may be T: each item reads and writes only its own kD^2 entries).
-// By thread ti of nt; returns this thread's part of |theta|_F^2.
+// lam_{b-1} Phi, both row-major: row (al s1), column (s2 ga).  With have_pre the
+// product B_b B_{b+1} is in T already.  By one warp, or (cta) by every thread of
+// the CTA; returns this thread's part of |theta|_F^2.  gs: 16 shared elements.
+//
+// Three passes of one element per thread each: product, gate, Schmidt values.
+// A thread that took a whole (al, ga) through all three left half the lanes idle
+// in its second round (36 pairs on 32 lanes at bonds of 6): 10,200 cycles an
+// update on 8 qubits, 5,200 in passes; 250,000 and 57,500 in the operator form.
 template <int kD>
-__device__ __noinline__ double theta_build(const TrajParams& p, const Lay& Y, unsigned char* slot, int b, const double2* G,
-                              bool adjoint, double2* T, double2* Phi, const double2* pre, int ti, int nt) {
-  constexpr int kI = kD / 2;
-  const int lstride = Y.L.chi;
+__device__ __noinline__ double theta_build(const TrajParams& p, const Lay& Y, unsigned char* slot, int b,
+                                           const double2* G, bool adjoint, double2* T, double2* Phi, bool have_pre,
+                                           double2* gs, bool cta) {
+  constexpr int kI = kD / 2, kDD = kD * kD;
+  const int ti = cta ? (int)threadIdx.x : (int)(threadIdx.x & 31), nt = cta ? (int)blockDim.x : 32;
   const int* D = slot_dims(slot);
   const int Dl = D[b], Dc = D[b + 1], Dr = D[b + 2];
-  const int n = kD * Dr;
+  const int n = kD * Dr, total = kD * Dl * n;
   const double2* sites = slot_sites(slot, Y.L);
-  const double* lam = slot_lam(slot, Y.L);
+  const double* lam = slot_lam(slot, Y.L) + (size_t)(b > 0 ? b - 1 : 0) * Y.L.chi;
   const double2* A = sites + Y.site_off[b];
   const double2* Bt = sites + Y.site_off[b + 1];
-
-  double2 g[16];
+  if (ti < 16) gs[ti] = adjoint ? cconj(G[(ti & 3) * 4 + (ti >> 2)]) : G[ti];
+  if (!have_pre) {
+#pragma unroll 1
+    for (int u = ti; u < total; u += nt) {
+      const int row = u / n, col = u - row * n;
+      double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 2
+      for (int be = 0; be < Dc; ++be) cfma(acc, A[(size_t)row * Dc + be], Bt[(size_t)be * n + col]);
+      T[u] = acc;
+    }
+  }
+  if (cta) __syncthreads(); else __syncwarp();
+#pragma unroll 1
+  for (int u = ti; u < total; u += nt) {
+    const int q = u / Dr, ga = u - q * Dr, al = q / kDD, ss = q - al * kDD;
+    const int s1 = ss / kD, s2 = ss - s1 * kD;
+    const double2* g = gs + ((s1 / kI) * 2 + s2 / kI) * 4;
+    const double2* t = T + ((size_t)al * kDD + (s1 % kI) * kD + s2 % kI) * Dr + ga;
+    double2 v = make_double2(0.0, 0.0);
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int p1 = 0; p1 < 2; ++p1)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) g[r * 4 + c] = adjoint ? cconj(G[c * 4 + r]) : G[r * 4 + c];
-
+      for (int p2 = 0; p2 < 2; ++p2) cfma(v, g[p1 * 2 + p2], t[(p1 * kI * kD + p2 * kI) * Dr]);
+    Phi[u] = v;
+  }
+  if (cta) __syncthreads(); else __syncwarp();
   double fro = 0.0;
 #pragma unroll 1
-  for (int it = ti; it < Dl * Dr; it += nt) {
-    const int al = it / Dr, ga = it - al * Dr;
-    double2 acc[kD * kD];   // (B_b B_{b+1})[al][s1][s2][ga] at s1 kD + s2
-    if (pre) {
-#pragma unroll
-      for (int q = 0; q < kD * kD; ++q) acc[q] = pre[((size_t)al * kD * kD + q) * Dr + ga];
-    } else {
-#pragma unroll
-      for (int q = 0; q < kD * kD; ++q) acc[q] = make_double2(0.0, 0.0);
-      const double2* ap = A + (size_t)(al * kD) * Dc;
-#pragma unroll 1
-      for (int be = 0; be < Dc; ++be) {
-        double2 av[kD], bv[kD];
-#pragma unroll
-        for (int q = 0; q < kD; ++q) {
-          av[q] = ap[(size_t)q * Dc + be];
-          bv[q] = Bt[(size_t)(be * kD + q) * Dr + ga];
-        }
-#pragma unroll
-        for (int q1 = 0; q1 < kD; ++q1)
-#pragma unroll
-          for (int q2 = 0; q2 < kD; ++q2) cfma(acc[q1 * kD + q2], av[q1], bv[q2]);
-      }
-    }
-    const double ll = (b > 0) ? lam[(size_t)(b - 1) * lstride + al] : 1.0;
-#pragma unroll
-    for (int s1 = 0; s1 < kD; ++s1)
-#pragma unroll
-      for (int s2 = 0; s2 < kD; ++s2) {
-        const int o1 = s1 / kI, i1 = s1 % kI, o2 = s2 / kI, i2 = s2 % kI;
-        const int row = o1 * 2 + o2;
-        double2 v = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int p1 = 0; p1 < 2; ++p1)
-#pragma unroll
-          for (int p2 = 0; p2 < 2; ++p2)
-            cfma(v, g[row * 4 + p1 * 2 + p2], acc[(p1 * kI + i1) * kD + p2 * kI + i2]);
-        const size_t idx = (size_t)(al * kD + s1) * n + s2 * Dr + ga;
-        Phi[idx] = v;
-        const double2 th = cscale(v, ll);
-        T[idx] = th;
-        fro += cabs2(th);
-      }
+  for (int u = ti; u < total; u += nt) {
+    const double ll = (b > 0) ? lam[u / (kDD * Dr)] : 1.0;
+    const double2 th = cscale(Phi[u], ll);
+    T[u] = th;
+    fro += cabs2(th);
   }
   return fro;
 }
@@ -381,7 +368,7 @@ __device__ __forceinline__ int upd_elems(int m, int n) { return m * n + svd_elem
 template <int kD>
 __device__ __noinline__ void two_site_update(const TrajParams& p, const Lay& Y, unsigned char* slot, int b,
                                              const double2* G, bool adjoint, bool record, bool count, WarpCtx& w,
-                                             const double2* pre = nullptr) {
+                                             bool have_pre = false) {
   const int lane = w.lane;
   const int* D = slot_dims(slot);
   const int m = kD * D[b], n = kD * D[b + 2];
@@ -389,7 +376,7 @@ __device__ __noinline__ void two_site_update(const TrajParams& p, const Lay& Y, 
   double2* Phi = upd_elems(m, n) <= p.slab_elems ? w.slab + svd_elems(m, n) : w.scratch;
   int4* X = reinterpret_cast<int4*>(w.slab + m * n);
   TNRC_TIC(t_c);
-  const double fro = warp_sum(theta_build<kD>(p, Y, slot, b, G, adjoint, T, Phi, pre, lane, 32));
+  const double fro = warp_sum(theta_build<kD>(p, Y, slot, b, G, adjoint, T, Phi, have_pre, w.small, false));
   __syncwarp();
   TNRC_TOC(w, 0, t_c);
   TNRC_TIC(t_j);
@@ -436,7 +423,7 @@ __device__ __forceinline__ WideHome wide_home(const TrajParams& p, int m, int n,
 template <int kD>
 __device__ __noinline__ void wide_update_cta(const TrajParams& p, const Lay& Y, unsigned char* slot, int b,
                                              const double2* G, bool adjoint, bool record, bool count, WarpCtx& w,
-                                             const double2* pre = nullptr) {
+                                             bool have_pre = false) {
   const int ti = threadIdx.x, nt = blockDim.x, warp = ti >> 5;
   const int* D = slot_dims(slot);
   const int m = kD * D[b], n = kD * D[b + 2];
@@ -444,7 +431,7 @@ __device__ __noinline__ void wide_update_cta(const TrajParams& p, const Lay& Y, 
   int4* X = reinterpret_cast<int4*>(h.X);
   WideShared* ws = w.wide;
   TNRC_TIC(t_c);
-  const double part = warp_sum(theta_build<kD>(p, Y, slot, b, G, adjoint, h.T, h.Phi, pre, ti, nt));
+  const double part = warp_sum(theta_build<kD>(p, Y, slot, b, G, adjoint, h.T, h.Phi, have_pre, w.cta_small, true));
   if (w.lane == 0) ws->part[warp] = part;
   __syncthreads();
   double fro = 0.0;
@@ -533,8 +520,7 @@ __device__ __forceinline__ double2* pair_theta(const TrajParams& p, const int* D
 template <int kD>
 __device__ __noinline__ void two_site_update_pair(const TrajParams& p, const Lay& Y, unsigned char* slot, int b1,
                                      const double2* G1, int b2, const double2* G2, bool adjoint, bool record,
-                                     bool count, WarpCtx& w, const double2* pre1 = nullptr,
-                                     const double2* pre2 = nullptr) {
+                                     bool count, WarpCtx& w, bool have_pre = false) {
   const int lane = w.lane;
   const int* D = slot_dims(slot);
   const int m1 = kD * D[b1], n1 = kD * D[b1 + 2], m2 = kD * D[b2], n2 = kD * D[b2 + 2];
@@ -543,8 +529,8 @@ __device__ __noinline__ void two_site_update_pair(const TrajParams& p, const Lay
   double2* T2 = w.slab + upd_elems(m1, n1);
   double2* Phi2 = T2 + m2 * n2;
   TNRC_TIC(t_c);
-  const double fro1 = warp_sum(theta_build<kD>(p, Y, slot, b1, G1, adjoint, T1, Phi1, pre1, lane, 32));
-  const double fro2 = warp_sum(theta_build<kD>(p, Y, slot, b2, G2, adjoint, T2, Phi2, pre2, lane, 32));
+  const double fro1 = warp_sum(theta_build<kD>(p, Y, slot, b1, G1, adjoint, T1, Phi1, have_pre, w.small, false));
+  const double fro2 = warp_sum(theta_build<kD>(p, Y, slot, b2, G2, adjoint, T2, Phi2, have_pre, w.small + 16, false));
   __syncwarp();
   TNRC_TOC(w, 0, t_c);
   const SvdBufs bf1{w.sig2, w.qn, w.perm, w.piv};
@@ -663,22 +649,13 @@ __device__ __noinline__ size_t pack_state(const TrajParams& p, const Lay& Y, con
 // Transfer-matrix steps of <c| . |a>.
 // Left:  Eout[b'][a'] = sum_{b,s,a} conj(c[b][s][b']) Ein[b][a] a[a][s][a']
 // Right: Eout[b][a]   = sum_{s,b',a'} conj(c[b][s][b']) Ein[b'][a'] a[a][s][a']
-// Run by a team of nt threads (thread ti of the team): one warp (nt = 32,
-// bar < 0: the warp synchronises itself) or several warps meeting at the
-// named barrier `bar`.  Every output element is summed by one thread in the
-// same order whatever the team, so the result does not depend on it.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void team_sync(int bar, int nt) {
-  if (bar < 0)
-    __syncwarp();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nt) : "memory");
-}
 
+// The left step of the final overlap, by one warp in FP64.
 template <int kD>
-__device__ __noinline__ void env_left_step(const double2* Ein, int Dcl, int Dal, const double2* c, int Dcr,
-                              const double2* a, int Dar, double2* tmp, double2* Eout, int ti, int nt = 32,
-                              int bar = -1) {
+__device__ __noinline__ void overlap_step(const double2* Ein, int Dcl, int Dal, const double2* c, int Dcr,
+                                          const double2* a, int Dar, double2* tmp, double2* Eout, int ti) {
+  const int nt = 32;
   const int w2 = kD * Dar;
 #pragma unroll 1
   for (int it = ti; it < Dcl * w2; it += nt) {
@@ -688,7 +665,7 @@ __device__ __noinline__ void env_left_step(const double2* Ein, int Dcl, int Dal,
     for (int al = 0; al < Dal; ++al) cfma(acc, Ein[be * Dal + al], a[(size_t)al * w2 + rest]);
     tmp[it] = acc;
   }
-  team_sync(bar, nt);
+  __syncwarp();
 #pragma unroll 1
   for (int it = ti; it < Dcr * Dar; it += nt) {
     const int bp = it / Dar, ap = it - bp * Dar;
@@ -700,36 +677,131 @@ __device__ __noinline__ void env_left_step(const double2* Ein, int Dcl, int Dal,
         cfmac(acc, c[(size_t)be * kD * Dcr + s * Dcr + bp], tmp[(size_t)be * w2 + s * Dar + ap]);
     Eout[it] = acc;
   }
-  team_sync(bar, nt);
+  __syncwarp();
 }
 
+// ---------------------------------------------------------------------------
+// The environments and the gate gradients of the costate sweep in fixed point.
+// They are sums over whole bonds that only the gradient reads, so one scale per
+// tensor keeps all that it needs (what the updates read stays FP64).  Every site
+// tensor of the two states is brought to integers once per layer, its largest
+// entry near 2^55; an environment carries the exponent of its own largest entry.
+// In FP64 (a complex multiply-add is four instructions of 64 cycles, in integers
+// twelve of five) these two took a third of a small evaluation.
+// ---------------------------------------------------------------------------
+struct EnvMem {
+  int4 *L, *R;       // environments, chi^2 elements per bond
+  int4 *c, *a;       // site tensors of the costate and of the forward state, at slot offsets
+  int *eL, *eR;      // exponents of the environments [N+1], real value = v 2^(e - 55)
+  int *ec, *ea;      // exponents of the site tensors [N]
+};
+__device__ __forceinline__ EnvMem env_mem(const TrajParams& p, int region) {
+  const size_t cc = (size_t)p.chi * p.chi, ne = (size_t)(p.N + 1) * cc;
+  EnvMem m;
+  m.L = reinterpret_cast<int4*>(p.env_scratch + (size_t)region * p.env_elems);
+  m.R = m.L + ne;
+  m.c = m.R + ne;
+  m.a = m.c + p.site_elems;
+  m.eL = reinterpret_cast<int*>(m.a + p.site_elems);
+  m.eR = m.eL + p.N + 1;
+  m.ec = m.eR + p.N + 1;
+  m.ea = m.ec + p.N + 1;
+  return m;
+}
+
+// Sum of products / 2^55 2^sh, |sh| <= 26.
+__device__ __forceinline__ long long fx_sum55(FxAcc s, int sh) {
+  const long long h = sh >= -1 ? s.h << (1 + sh) : s.h >> (-1 - sh);
+  return h + ((s.x + (1ll << (26 - sh))) >> (27 - sh));
+}
+
+// A site tensor (cnt entries) to integers, by one warp.
+static __device__ __noinline__ void site_to_fx(const double2* src, int cnt, int4* dst, int* ex, int lane) {
+  int mx = 0;
+#pragma unroll 1
+  for (int e = lane; e < cnt; e += 32) {
+    const double2 v = src[e];
+    mx = max(mx, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
+  }
+  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
+  const int x = (mx >> 20) - 1022;
+#pragma unroll 1
+  for (int e = lane; e < cnt; e += 32) dst[e] = fx_from_double2(src[e], 55 - x);
+  if (lane == 0) *ex = x;
+}
+
+// Every thread of the CTA: both states' sites, and the outermost environments.
 template <int kD>
-__device__ __noinline__ void env_right_step(const double2* Ein, int Dcr, int Dar, const double2* c, int Dcl,
-                               const double2* a, int Dal, double2* tmp, double2* Eout, int ti, int nt = 32,
-                               int bar = -1) {
-  const int w2 = kD * Dal;
+__device__ __noinline__ void layer_to_fx(const TrajParams& p, const Lay& Y, const unsigned char* cslot,
+                                         const StateView av, WarpCtx& w) {
+  const EnvMem m = env_mem(p, w.region);
+  const int* Dc = slot_dims(cslot);
+  const double2* cs = slot_sites(cslot, Y.L);
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll 1
-  for (int it = ti; it < Dcr * w2; it += nt) {
-    const int bp = it / w2, rest = it - bp * w2;
-    const int s = rest / Dal, al = rest - s * Dal;
-    double2 acc = make_double2(0.0, 0.0);
-#pragma unroll 1
-    for (int ap = 0; ap < Dar; ++ap) cfma(acc, Ein[bp * Dar + ap], a[(size_t)al * kD * Dar + s * Dar + ap]);
-    tmp[it] = acc;
+  for (int u = warp; u < 2 * p.N; u += nw) {
+    const int i = u >> 1, off = Y.site_off[i];
+    if (u & 1)
+      site_to_fx(av.sites + av.off[i], av.D[i] * kD * av.D[i + 1], m.a + off, m.ea + i, w.lane);
+    else
+      site_to_fx(cs + off, Dc[i] * kD * Dc[i + 1], m.c + off, m.ec + i, w.lane);
   }
-  team_sync(bar, nt);
+  if (threadIdx.x == 0) {
+    const int4 one = make_int4(1 << 27, 0, 0, 0);
+    m.L[0] = one;
+    m.R[(size_t)p.N * p.chi * p.chi] = one;
+    m.eL[0] = 0;
+    m.eR[p.N] = 0;
+    for (int t = 0; t < 6; ++t) w.wide->ring[t] = 0;
+  }
+}
+
+// The team of one sweep meets at its named barrier.
+__device__ __forceinline__ void team_sync(int team, int nt) {
+  if (team == 0)
+    asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
+  else
+    asm volatile("bar.sync 2, %0;" ::"r"(nt) : "memory");
+}
+
+// One step by thread ti of nt.  The first product takes the shift sh that brings
+// the environment's largest entry to 2^55; the largest entry of the result (as
+// its bit length) is left in *bits.  Left (team 0): k runs over the left bonds.
+template <int kD>
+__device__ __noinline__ void env_step(int team, const int4* Ein, int D1, int K1, const int4* c, int cs1, int cs2,
+                                      const int4* a, int as1, int as2, int D2, int Da2, int4* tmp, int4* Eout, int sh,
+                                      int* bits, int ti, int nt) {
+  // tmp[i][s][y] = sum_k Ein[i][k] a(k, s, y), i < D1, k < K1, y < Da2; a(k, s, y) at
+  // k as1 + s Da' + y as2 (s stride: Da2 on the left, K1 on the right)
+  const int as_s = team == 0 ? Da2 : K1, w2 = kD * Da2;
 #pragma unroll 1
-  for (int it = ti; it < Dcl * Dal; it += nt) {
-    const int be = it / Dal, al = it - be * Dal;
-    double2 acc = make_double2(0.0, 0.0);
+  for (int it = ti; it < D1 * w2; it += nt) {
+    const int i = it / w2, rest = it - i * w2, s = rest / Da2, y = rest - s * Da2;
+    const int4* ap = a + s * as_s + y * as2;
+    FxAcc re{0, 0}, im{0, 0};
+#pragma unroll 2
+    for (int k = 0; k < K1; ++k) fx_cmac(re, im, Ein[i * K1 + k], ap[k * as1]);
+    tmp[it] = fx_pack(fx_sum55(re, sh), fx_sum55(im, sh));
+  }
+  team_sync(team, nt);
+  // Eout[x][y] = sum_{i,s} conj(c(i, s, x)) tmp[i][s][y], c(i, s, x) at i cs1 + s cs' + x cs2
+  const int cs_s = team == 0 ? D2 : D1;
+  long long top = 0;
 #pragma unroll 1
-    for (int bp = 0; bp < Dcr; ++bp)
+  for (int it = ti; it < D2 * Da2; it += nt) {
+    const int x = it / Da2, y = it - x * Da2;
+    FxAcc re{0, 0}, im{0, 0};
+#pragma unroll 1
+    for (int i = 0; i < D1; ++i)
 #pragma unroll
-      for (int s = 0; s < kD; ++s)
-        cfmac(acc, c[(size_t)be * kD * Dcr + s * Dcr + bp], tmp[(size_t)bp * w2 + s * Dal + al]);
-    Eout[it] = acc;
+      for (int s = 0; s < kD; ++s) fx_cmacc(re, im, c[i * cs1 + s * cs_s + x * cs2], tmp[i * w2 + s * Da2 + y]);
+    const long long vr = fx_sum55(re, 0), vi = fx_sum55(im, 0);
+    top |= (vr < 0 ? -vr : vr) | (vi < 0 ? -vi : vi);
+    Eout[it] = fx_pack(vr, vi);
   }
-  team_sync(bar, nt);
+  const int b = (int)__reduce_max_sync(0xffffffffu, (unsigned)(64 - __clzll(top)));
+  if ((threadIdx.x & 31) == 0) atomicMax(bits, b);
+  team_sync(team, nt);
 }
 
 // <t|a> by one warp.
@@ -748,8 +820,8 @@ __device__ __noinline__ double2 warp_overlap(const TrajParams& p, const Lay& Yt,
   __syncwarp();
 #pragma unroll 1
   for (int i = 0; i < p.N; ++i) {
-    env_left_step<kD>(E0, Dt[i], Da[i], ts + Yt.site_off[i], Dt[i + 1], as + Ya.site_off[i], Da[i + 1], tmp, E1,
-                      w.lane);
+    overlap_step<kD>(E0, Dt[i], Da[i], ts + Yt.site_off[i], Dt[i + 1], as + Ya.site_off[i], Da[i + 1], tmp, E1,
+                     w.lane);
     double2* x = E0;
     E0 = E1;
     E1 = x;
@@ -820,65 +892,78 @@ static __device__ __noinline__ void order_layer(const TrajParams& p, const int* 
 // ---------------------------------------------------------------------------
 template <int kD>
 __device__ __noinline__ void layer_envs(const TrajParams& p, const Lay& Y, const unsigned char* cslot, const StateView av,
-                           WarpCtx& w, int warp) {
-  const int N = p.N, chi = p.chi;
-  const size_t cc = (size_t)chi * chi;
+                                        WarpCtx& w, int warp) {
+  const int N = p.N;
+  const size_t cc = (size_t)p.chi * p.chi;
   const int* Dc = slot_dims(cslot);
   const int* Da = av.D;
-  const double2* cs = slot_sites(cslot, Y.L);
-  const double2* as = av.sites;
-  const int* so = Y.site_off;   // costate slot offsets
-  const int* ao = av.off;       // forward-state offsets
-  double2* Lbuf = p.env_scratch + (size_t)w.region * 2 * (N + 1) * cc;
-  double2* Rbuf = Lbuf + (size_t)(N + 1) * cc;
-  const int lane = w.lane;
+  const int* off = Y.site_off;
+  const EnvMem m = env_mem(p, w.region);
 
   // left environments L_i (sites < i) for i <= N-2 by the even warps, right
   // R_i (sites >= i) for i >= 2 by the odd warps: each sweep is sequential
-  // over the sites, so each step is shared by its team of warps (named
-  // barriers 1 and 2); the step's intermediate (at most Dc x kD Da) sits in
-  // the team's first warp's shared slab when it fits, else in its scratch
+  // over the sites, so each step is shared by its team of warps; the step's
+  // intermediate (at most Dc x kD Da) sits in the team's first warp's shared
+  // slab when it fits, else in its scratch.  Each element is summed by one
+  // thread, so the result does not depend on the team.
   TNRC_TIC(t_e);
   const int team = warp & 1;                               // 0: left, 1: right
   const int nt = 32 * (team == 0 ? (p.warps + 1) / 2 : p.warps / 2);
-  const int ti = (warp >> 1) * 32 + lane;
-  double2* lead_slab = w.slab - (size_t)(warp - team) * p.slab_elems;
-  double2* lead_scratch = w.scratch - (size_t)(warp - team) * p.scratch_elems;
-  const bool lead = warp == team;
-  if (team == 0) {
+  const int ti = (warp >> 1) * 32 + w.lane;
+  int4* lead_slab = reinterpret_cast<int4*>(w.slab - (size_t)(warp - team) * p.slab_elems);
+  int4* lead_scratch = reinterpret_cast<int4*>(w.scratch - (size_t)(warp - team) * p.scratch_elems);
+  int* ring = w.wide->ring + 3 * team;   // largest entries of three steps in turn
+  int sh = 0, e = 0;
 #pragma unroll 1
-    for (int i = 0; i + 1 <= N - 2; ++i) {
-      double2* tmp = (Dc[i] * kD * Da[i + 1] <= p.slab_elems) ? lead_slab : lead_scratch;
-      env_left_step<kD>(Lbuf + i * cc, Dc[i], Da[i], cs + so[i], Dc[i + 1], as + ao[i], Da[i + 1],
-                        tmp, Lbuf + (i + 1) * cc, ti, nt, 1);
-      if (lead) w.alg += 8ull * kD * Da[i + 1] * (unsigned long long)(Dc[i] * Da[i] + Dc[i + 1] * Dc[i]);
+  for (int t = 0; t < N - 2; ++t) {
+    const int i = team == 0 ? t : N - 1 - t;               // the site taken in
+    int* bits = ring + t % 3;
+    const int cl = Dc[i], cr = Dc[i + 1], al = Da[i], ar = Da[i + 1];
+    const int n1 = kD * (team == 0 ? cl * ar : cr * al);
+    int4* tmp = n1 <= p.slab_elems ? lead_slab : lead_scratch;
+    const int4 *c = m.c + off[i], *a = m.a + off[i];
+    if (team == 0)
+      env_step<kD>(0, m.L + i * cc, cl, al, c, kD * cr, 1, a, kD * ar, 1, cr, ar, tmp, m.L + (i + 1) * cc, sh, bits, ti,
+                   nt);
+    else
+      env_step<kD>(1, m.R + (i + 1) * cc, cr, ar, c, 1, kD * cr, a, 1, kD * ar, cl, al, tmp, m.R + i * cc, sh, bits, ti,
+                   nt);
+    e += m.ec[i] + m.ea[i] - sh;
+    const int b = *bits;
+    sh = b > 0 ? max(-26, min(26, 55 - b)) : 0;
+    if (ti == 0) {
+      (team == 0 ? m.eL : m.eR)[team == 0 ? i + 1 : i] = e;
+      ring[(t + 2) % 3] = 0;   // read by every thread before the barrier within this step
     }
-  } else {
-#pragma unroll 1
-    for (int i = N - 1; i >= 2; --i) {
-      double2* tmp = (Dc[i + 1] * kD * Da[i] <= p.slab_elems) ? lead_slab : lead_scratch;
-      env_right_step<kD>(Rbuf + (size_t)(i + 1) * cc, Dc[i + 1], Da[i + 1], cs + so[i], Dc[i],
-                         as + ao[i], Da[i], tmp, Rbuf + (size_t)i * cc, ti, nt, 2);
-      if (lead) w.alg += 8ull * kD * Da[i] * (unsigned long long)(Dc[i + 1] * Da[i + 1] + Dc[i] * Dc[i + 1]);
-    }
+    if (ti == 0) w.alg += 8ull * n1 * (unsigned long long)(team == 0 ? al : ar) + 8ull * kD * cl * cr * (team == 0 ? ar : al);
   }
   TNRC_TOC(w, 4, t_e);
+}
+
+// out[i][j] = sum_k A[i K + k] B(k, j), M x J outputs, B(k, j) at k bk + j bj.
+static __device__ __noinline__ void fx_gemm(const int4* A, const int4* B, int M, int K, int J, int bk, int bj, int4* out,
+                                            int ti, int nt) {
+#pragma unroll 1
+  for (int it = ti; it < M * J; it += nt) {
+    const int i = it / J, j = it - i * J;
+    FxAcc re{0, 0}, im{0, 0};
+#pragma unroll 2
+    for (int k = 0; k < K; ++k) fx_cmac(re, im, A[i * K + k], B[k * bk + j * bj]);
+    out[it] = fx_pack(fx_sum55(re, 0), fx_sum55(im, 0));
+  }
 }
 
 template <int kD>
 __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, const unsigned char* cslot, const StateView av,
                               int s, int l, int b, double2 wO, double* gsp_row, WarpCtx& w, double2* Wc, bool cta) {
   constexpr int kDD = kD * kD, kI = kD / 2;
-  const int N = p.N, chi = p.chi;
+  const int chi = p.chi;
   const size_t cc = (size_t)chi * chi;
   const int* Dc = slot_dims(cslot);
   const int* Da = av.D;
   const double2* cs = slot_sites(cslot, Y.L);
-  const double2* as = av.sites;
   const int* so = Y.site_off;
-  const int* ao = av.off;
-  const double2* Lbuf = p.env_scratch + (size_t)w.region * 2 * (N + 1) * cc;
-  const double2* Rbuf = Lbuf + (size_t)(N + 1) * cc;
+  const EnvMem em = env_mem(p, w.region);
   const int lane = w.lane;
   const int ti = cta ? (int)threadIdx.x : lane, nt = cta ? (int)blockDim.x : 32;
   auto sync = [&]() {
@@ -890,10 +975,6 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
   TNRC_TIC(t_g);
   const int dcl = Dc[b], dcm = Dc[b + 1], dcr = Dc[b + 2];
   const int dal = Da[b], dam = Da[b + 1], dar = Da[b + 2];
-  const double2* L = Lbuf + (size_t)b * cc;
-  const double2* R = Rbuf + (size_t)(b + 2) * cc;
-  const double2* a0 = as + ao[b];
-  const double2* a1 = as + ao[b + 1];
   const double2* c0 = cs + so[b];
   const double2* c1 = cs + so[b + 1];
   // the costate product c_b c_{b+1} is shared with the bond's costate update
@@ -901,26 +982,22 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
   if (ti < 32)
     w.alg += 8ull * dcl * (kD * dam * dal + kDD * dar * dam + kDD * dcr * dar +
                            (unsigned long long)kDD * kDD * dcr) + 2048ull;
-  // Wc = c_b c_{b+1} [dcl][kD^2][dcr] at Wc (theta's home); the other three
-  // intermediates packed at their actual sizes right after it in the shared
-  // slab when they fit there, else in global scratch past theta's room
+  // Wc = c_b c_{b+1} [dcl][kD^2][dcr] at Wc (theta's home), in FP64 for the update
+  // that takes it over; the integer intermediates packed at their actual sizes
+  // right after it in the shared slab when they fit there, else in global
+  // scratch past theta's room
   const int n1 = dcl * kD * dam, n2 = dcl * kDD * dar, n3 = dcl * kDD * dcr;
   double2* slab = cta ? w.cta_slab : w.slab;
   const int slab_elems = cta ? p.cta_slab_elems : p.slab_elems;
   const bool wc_in_slab = Wc >= slab && Wc < slab + slab_elems;
-  double2* U1 = (wc_in_slab && (Wc - slab) + n3 + n1 + n2 + n3 <= slab_elems)
-                    ? Wc + n3
-                    : (cta ? w.cta_scratch : w.scratch) + (size_t)2 * kDD * chi * chi;   // [dcl][kD][dam]
-  double2* U2 = U1 + n1;                          // [dcl][kD^2][dar]
-  double2* U3 = U2 + n2;                          // [dcl][kD^2][dcr]
-#pragma unroll 1
-  for (int it = ti; it < dcl * kD * dam; it += nt) {
-    const int be = it / (kD * dam), rest = it - be * kD * dam;
-    double2 acc = make_double2(0.0, 0.0);
-#pragma unroll 1
-    for (int al = 0; al < dal; ++al) cfma(acc, L[be * dal + al], a0[(size_t)al * kD * dam + rest]);
-    U1[it] = acc;
-  }
+  int4* U1 = reinterpret_cast<int4*>((wc_in_slab && (Wc - slab) + n3 + n1 + n2 + 2 * n3 <= slab_elems)
+                                         ? Wc + n3
+                                         : (cta ? w.cta_scratch : w.scratch) + (size_t)2 * kDD * chi * chi);
+  int4* U2 = U1 + n1;   // U1 [dcl][kD][dam], U2 [dcl][kD^2][dar]
+  int4* U3 = U2 + n2;   // [dcl][kD^2][dcr]
+  int4* Wi = U3 + n3;   // Wc in integers
+  const int ew = em.ec[b] + em.ec[b + 1] + 2;   // |Wc| < 2^ew with room to spare
+  fx_gemm(em.L + (size_t)b * cc, em.a + so[b], dcl, dal, kD * dam, kD * dam, 1, U1, ti, nt);
 #pragma unroll 1
   for (int it = ti; it < dcl * kDD * dcr; it += nt) {
     const int be = it / (kDD * dcr), rest = it - be * kDD * dcr;
@@ -931,31 +1008,12 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
     for (int b1 = 0; b1 < dcm; ++b1)
       cfma(acc, c0[(size_t)be * kD * dcm + s1 * dcm + b1], c1[(size_t)b1 * kD * dcr + s2 * dcr + b2]);
     Wc[it] = acc;
+    Wi[it] = fx_from_double2(acc, 55 - ew);
   }
   sync();
-#pragma unroll 1
-  for (int it = ti; it < dcl * kDD * dar; it += nt) {
-    const int be = it / (kDD * dar), rest = it - be * kDD * dar;
-    const int ss = rest / dar, a2 = rest - ss * dar;
-    const int s1 = ss / kD, s2 = ss % kD;
-    double2 acc = make_double2(0.0, 0.0);
-#pragma unroll 1
-    for (int a1i = 0; a1i < dam; ++a1i)
-      cfma(acc, U1[(size_t)be * kD * dam + s1 * dam + a1i], a1[(size_t)a1i * kD * dar + s2 * dar + a2]);
-    U2[it] = acc;
-  }
+  fx_gemm(U1, em.a + so[b + 1], dcl * kD, dam, kD * dar, kD * dar, 1, U2, ti, nt);
   sync();
-#pragma unroll 1
-  for (int it = ti; it < dcl * kDD * dcr; it += nt) {
-    const int be = it / (kDD * dcr), rest = it - be * kDD * dcr;
-    const int ss = rest / dcr, b2 = rest - ss * dcr;
-    double2 acc = make_double2(0.0, 0.0);
-    const double2* u2 = U2 + (size_t)be * kDD * dar + ss * dar;
-    const double2* rr = R + (size_t)b2 * dar;
-#pragma unroll 1
-    for (int a2 = 0; a2 < dar; ++a2) cfma(acc, u2[a2], rr[a2]);
-    U3[it] = acc;
-  }
+  fx_gemm(U2, em.R + (size_t)(b + 2) * cc, dcl * kDD, dar, dcr, 1, dar, U3, ti, nt);
   sync();
   // rho[o'][o] = sum_{i1,i2} sum_{be,b2} U3[be][s'][b2] conj(Wc[be][s][b2]) over the
   // two-site out indices o (the in indices, if any, traced out: the gate acts
@@ -965,26 +1023,26 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
   {
     const int parts = cta ? 8 : 2;
     double2* sums = cta ? w.cta_small : w.small;   // at least two warps' 64 elements
+    const int e = em.eL[b] + em.ea[b] + em.ea[b + 1] + em.eR[b + 2] + ew;
 #pragma unroll 1
     for (int it = ti; it < 16 * parts; it += nt) {
       const int o = it & 15, part = it >> 4;
       const int op = o >> 2, oq = o & 3;
-      double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int i1 = 0; i1 < kI; ++i1)
-#pragma unroll
-        for (int i2 = 0; i2 < kI; ++i2) {
-          const int sp = ((op >> 1) * kI + i1) * kD + (op & 1) * kI + i2;
-          const int sq = ((oq >> 1) * kI + i1) * kD + (oq & 1) * kI + i2;
+      FxAcc re{0, 0}, im{0, 0};
 #pragma unroll 1
-          for (int be = part; be < dcl; be += parts) {
-            const double2* u = U3 + (size_t)be * kDD * dcr + sp * dcr;
-            const double2* wv = Wc + (size_t)be * kDD * dcr + sq * dcr;
+      for (int ii = 0; ii < kI * kI; ++ii) {
+        const int i1 = ii / kI, i2 = ii % kI;
+        const int sp = ((op >> 1) * kI + i1) * kD + (op & 1) * kI + i2;
+        const int sq = ((oq >> 1) * kI + i1) * kD + (oq & 1) * kI + i2;
 #pragma unroll 1
-            for (int b2 = 0; b2 < dcr; ++b2) cfmac(acc, wv[b2], u[b2]);
-          }
+        for (int be = part; be < dcl; be += parts) {
+          const int4* u = U3 + (size_t)be * kDD * dcr + sp * dcr;
+          const int4* wv = Wi + (size_t)be * kDD * dcr + sq * dcr;
+#pragma unroll 1
+          for (int b2 = 0; b2 < dcr; ++b2) fx_cmacc(re, im, wv[b2], u[b2]);
         }
-      sums[it] = acc;
+      }
+      sums[it] = make_double2(fx_scale((double)fx_sum55(re, 0), e - 55), fx_scale((double)fx_sum55(im, 0), e - 55));
     }
     sync();
     if (ti < 16) {
@@ -998,19 +1056,25 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
     }
     __syncwarp();
   }
-  // dO/du_q = tr(Q_q rho) = sum_ij Q_q[i][j] rho[j][i]: lane q takes control q
-  const LayerGate& lg = layer_rec(p, s, l, b);
-  const int nq = lg.nq;
-  if (ti < nq) {
-    const double2* Q = lg.Q[ti];
-    double2 v = make_double2(0.0, 0.0);
+  // dO/du_q = tr(Q_q rho) = sum_ij Q_q[i][j] rho[j][i]: control q by four lanes,
+  // one row i each
+  if (ti < 32) {
+    const LayerGate& lg = layer_rec(p, s, l, b);
+    const int nq = lg.nq;
+#pragma unroll 1
+    for (int q0 = 0; q0 < nq; q0 += 8) {
+      const int q = q0 + (lane >> 2), i = lane & 3;
+      double2 v = make_double2(0.0, 0.0);
+      if (q < nq) {
+        const double2* Q = lg.Q[q] + i * 4;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) cfma(v, Q[i * 4 + j], rho[j * 4 + i]);
-    // explicit fma: this function is inlined into both history modes, which
-    // must round identically
-    gsp_row[lg.slot[ti]] += 2.0 * fma(wO.x, v.x, wO.y * v.y);
+        for (int j = 0; j < 4; ++j) cfma(v, Q[j], rho[j * 4 + i]);
+      }
+      double t = fma(wO.x, v.x, wO.y * v.y);
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      if (q < nq && i == 0) gsp_row[lg.slot[q]] += 2.0 * t;
+    }
   }
   sync();
   TNRC_TOC(w, 5, t_g);
@@ -1145,7 +1209,7 @@ __device__ __noinline__ void costate_group(const TrajParams& p, const Lay& Y, un
     bond_gradient<kD>(p, Y, cslot, av, s, l, b1, wO, gsp_row, w, th1, false);
     bond_gradient<kD>(p, Y, cslot, av, s, l, b2, wO, gsp_row, w, th2, false);
     two_site_update_pair<kD>(p, Y, cslot, b1, layer_rec(p, s, l, b1).G, b2, layer_rec(p, s, l, b2).G, true, false,
-                             true, w, th1, th2);
+                             true, w, true);
     return;
   }
 #pragma unroll 1
@@ -1153,7 +1217,7 @@ __device__ __noinline__ void costate_group(const TrajParams& p, const Lay& Y, un
     const int b = q == 0 ? b1 : b2;
     if (b < 0) break;
     bond_gradient<kD>(p, Y, cslot, av, s, l, b, wO, gsp_row, w, w.slab, false);
-    two_site_update<kD>(p, Y, cslot, b, layer_rec(p, s, l, b).G, true, false, true, w, w.slab);
+    two_site_update<kD>(p, Y, cslot, b, layer_rec(p, s, l, b).G, true, false, true, w, true);
   }
 }
 
@@ -1173,13 +1237,8 @@ __device__ void costate_layer(const TrajParams& p, const Lay& Y, unsigned char* 
   int nb = (p.N - 1 - parity + 1) / 2;
   const int lane = w.lane;
   const int* Dc = slot_dims(cslot);
-  const size_t cc = (size_t)p.chi * p.chi;
   if (warp == p.warps - 1) order_layer(p, Dc, parity, w);
-  if (lane == 0 && warp == 0) {
-    double2* Lbuf = p.env_scratch + (size_t)w.region * 2 * (p.N + 1) * cc;
-    Lbuf[0] = make_double2(1.0, 0.0);
-    Lbuf[(size_t)(2 * p.N + 1) * cc] = make_double2(1.0, 0.0);   // R_N
-  }
+  layer_to_fx<kD>(p, Y, cslot, av, w);
   __syncthreads();
   layer_envs<kD>(p, Y, cslot, av, w, warp);
   __syncthreads();
@@ -1188,7 +1247,7 @@ __device__ void costate_layer(const TrajParams& p, const Lay& Y, unsigned char* 
       double2* th = wide_home<kD>(p, kD * Dc[b], kD * Dc[b + 2], w).T;
       bond_gradient<kD>(p, Y, cslot, av, s, l, b, wO, gsp_row, w, th, true);
       __syncthreads();
-      wide_update_cta<kD>(p, Y, cslot, b, layer_rec(p, s, l, b).G, true, false, true, w, th);
+      wide_update_cta<kD>(p, Y, cslot, b, layer_rec(p, s, l, b).G, true, false, true, w, true);
     });
   for (;;) {
     int e = 0;
