@@ -151,7 +151,7 @@ TNRC_HD long long fx_rsqrt(long long N) {
 struct FxRot {
   Fx c, s2x, s2y, s3x, s3y;
   int ka, kb;
-  float t;   // tangent of the angle
+  float s2;   // sin^2 of the angle
 };
 
 TNRC_HD void fx_rotation(long long aa, long long bb, long long abr, long long abi, int de, float af, float bf,
@@ -166,19 +166,20 @@ TNRC_HD void fx_rotation(long long aa, long long bb, long long abr, long long ab
   } else {
     D = bf * fx_pow2f(de) - af * fx_pow2f(-de);
   }
-  const float iab = fx_rsqrtf(ab2);
-  const float aab = ab2 * iab;
-  const float Da = fabsf(D), two = 2.0f * aab;
-  const float inv = fx_rcpf(fmaxf(Da, two));
-  const float dn = Da * inv, an = two * inv;
-  const float h2 = dn * dn + an * an;
-  const float t = an * fx_rcpf(dn + h2 * fx_rsqrtf(h2));
-  const float c0 = fx_rsqrtf(1.0f + t * t);
-  const float f = copysignf(t * c0 * iab, D);
+  // cos 2theta = |D| w, w = 1 / sqrt(D^2 + 4 |ab|^2), c = sqrt((1 + cos 2theta) /
+  // 2), s e^{i phi} = sign(D) w / c ab, scaled by inv against overflow: three
+  // dependent reciprocals and roots
+  const float inv = fx_rcpf(fmaxf(fabsf(D), 2.0f * (fabsf(xr) + fabsf(xi))));
+  const float dn = fabsf(D) * inv, an2 = 4.0f * ab2 * inv * inv;
+  const float w = fx_rsqrtf(fmaf(dn, dn, an2));
+  const float hq = fmaf(0.5f, dn * w, 0.5f);   // c^2
+  const float rc = fx_rsqrtf(hq);
+  const float c0 = hq * rc;
+  const float f = copysignf(inv * w * rc, D);
   float sx = f * xr, sy = f * xi;
-  R.t = t;
+  R.s2 = sx * sx + sy * sy;
   const float p = fx_pow2f(de), q = fx_pow2f(-de);
-  float dt = copysignf(t * aab, D);
+  float dt = ab2 * f * rc;   // tan theta |ab|, with the sign of D
   if (!(fmaxf(fabsf(sx), fabsf(sy)) * fmaxf(p, q) < 7.5f)) {
     // scales out of date by more than the limbs hold (cannot happen while the
     // shifts below keep up): refresh them, rotate in a later round

@@ -480,7 +480,7 @@ __device__ __noinline__ int fx_qr_cta(double2* T, int4* Pw, int m, int n, double
 // products and both norms of a pair are formed in every round (the integer
 // products are cheap, carried norms would need FP64), the angle in FP32
 // (fx_rotation).  The last sweep is one whose rotations all had |cos| max(|cos|,
-// tan) <= 1e-16, with |cos| between the pair's columns and tan of the angle:
+// sin) <= 1e-16, with |cos| between the pair's columns and sin of the angle:
 // what a rotation puts back into the pairs before it in the sweep is that
 // product, and what the FP32 angle leaves of its own pair is 1e-7 |cos|.
 // ---------------------------------------------------------------------------
@@ -549,7 +549,7 @@ __device__ __forceinline__ void fx_pair(const FxMem<SH>& X, int ldx, int n, int 
     FxRot R;
     fx_rotation(aa, bb, abr, abi, ej - ei, af, bf, xr, xi, ab2, R);
     rotated = 1;
-    large |= (ab2 * fmaxf(ab2, R.t * R.t * pab) > 1e-32f * pab * pab) ? 1 : 0;
+    large |= (ab2 * fmaxf(ab2, R.s2 * pab) > 1e-32f * pab * pab) ? 1 : 0;
     const Fx n2x = fx_neg(R.s2x), n2y = fx_neg(R.s2y), n3y = fx_neg(R.s3y);
 #pragma unroll 1
     for (int row = lig; row < n; row += 1 << lg) {

@@ -10,7 +10,8 @@
 //            Eq. circuit two layers per step (odd bonds; even bonds with the
 //            single-site rotations folded in).  Every two-site gate is
 //            followed by the truncated SVD; the warps of the CTA share the
-//            disjoint bonds of a layer, largest first.
+//            disjoint bonds of a layer, largest first, and work together on a
+//            bond that is a large part of its layer.
 //   overlap  (Sec. II state form): O = <t_p | a(T)> by a transfer-matrix sweep.
 //   gradient (App. A): the costate b_l = L_{l+1}^dag .. L_L^dag t is propagated
 //            backwards with the same truncated update; for every gate of layer
@@ -21,6 +22,15 @@
 //            checkpoints when the history does not fit).
 // Each trajectory writes its own O and its own gradient row, so results do not
 // depend on which CTA ran it or on what else ran in the launch.
+//
+// What bounds it: with the SVDs, the environments and the gradients in integers
+// (fx.cuh) the FP64 pipe is 13 % busy on the 50-qubit benchmark and DRAM at 1 %;
+// a warp waits for the results of its own instructions (fixed latencies a third
+// of the stalls, then shared and L2 loads, barriers and instruction fetch), two
+// warps to a scheduler, which the 220 KB of shared memory for theta and
+// R^dagger allow.  Every function is out of line and no runtime loop unrolled:
+// inlined and unrolled the kernel overran the instruction cache, which cost
+// 45 % of the stalls (50-qubit CNOT, 304 trajectories: 742 ms, then 386 ms).
 #pragma once
 #include "svd_fx.cuh"
 
@@ -35,9 +45,9 @@ struct WarpCtx {
   double2* slab;       // shared, slab_elems
   double2* scratch;    // global, scratch_elems
   double* sig2;        // shared, kMaxDim
-  double* qn;          // shared, kMaxDim (column norms of the pivoted QR)
+  double* qn;          // shared, kMaxDim (SvdBufs)
   int* perm;           // shared, kMaxDim
-  int* piv;            // shared, kMaxDim (column pivots of the QR)
+  int* piv;            // shared, kMaxDim
   double2* small;      // shared, 64 complex (four 4x4 matrices)
   int lane;
   long long sweeps;
@@ -91,12 +101,14 @@ __device__ __forceinline__ const LayerGate& layer_rec(const TrajParams& p, int s
 // ---------------------------------------------------------------------------
 // Two-site update of bond b: theta = lam_{b-1} G (B_b B_{b+1}), truncated SVD,
 // B_{b+1} <- Y_k^dag, B_b <- Phi Y_k / |S_k|, lam_b <- S_k / |S_k|.
-// The SVD: theta P = Q R by pivoted QR (Q not formed; R has r rows, r the
-// numerical rank), then one-sided Jacobi on the r columns of R^dagger:
-// R^dagger V = Z S, so theta = (Q V) S (P Z)^dagger and Y = P Z.
+// The SVD (svd_fx.cuh, in integers): theta = Q R by pivoted Gram-Schmidt (Q not
+// kept; R has r rows, r the numerical rank), then one-sided Jacobi on the r
+// columns of R^dagger: R^dagger V = Z S, so theta = (Q V) S Z^dagger and Y = Z.
 // ---------------------------------------------------------------------------
-// Per-matrix work arrays of the SVD (shared, per warp): squared singular
-// values, column norms (later 1 / sigma), rank order, QR column pivots.
+// Per-matrix work arrays of the SVD (shared, per warp): squared singular values
+// (row exponents during the QR), column norms of the QR and then the columns'
+// exponents, exponents of R^dagger and then the rank order, QR column order and
+// then the columns' shifts.
 struct SvdBufs {
   double* sig2;
   double* qn;
@@ -483,10 +495,8 @@ __device__ __noinline__ void wide_update_cta(const TrajParams& p, const Lay& Y, 
   TNRC_TOC(w, 3, t_w);
 }
 
-#ifndef TNRC_PAIR_SIDE
-#define TNRC_PAIR_SIDE 64
-#endif
-constexpr int kPairSide = TNRC_PAIR_SIDE;
+constexpr int kPairSide = 64;
+
 // Bonds a warp takes at a time.  Two, with small ones as a pair, where a layer
 // has more bonds than an SM's eight warps twice over; one below that, where
 // pairs would leave warps without a bond (8 qubits, 4 bonds a layer: 5.9 ms
@@ -505,18 +515,18 @@ __device__ __forceinline__ bool pair_fits(const TrajParams& p, const int* D, int
          m2 <= kPairSide && n2 <= kPairSide;
 }
 
-// Where a pair update keeps its two thetas in the slab: T1 at 0, Phi1 at
-// m1 n1, T2 at 2 m1 n1, Phi2 after T2.
+// Where a pair update keeps its two thetas in the slab: theta, Phi, R^dagger and
+// the pivot column of the first, then the same of the second.
 template <int kD>
 __device__ __forceinline__ double2* pair_theta(const TrajParams& p, const int* D, int b1, int which, WarpCtx& w) {
   return which == 0 ? w.slab : w.slab + upd_elems(kD * D[b1], kD * D[b1 + 2]);
 }
 
 // Two two-site updates (bonds b1, b2 of one layer, disjoint sites) by one
-// warp: thetas built one after the other, then the pivoted QR and the Jacobi
-// of both at once on the two half-warps, then ranks and splits one after the
-// other.  The same arithmetic per bond as two_site_update, in another lane
-// arrangement (so the same results up to the order of sums).
+// warp: thetas built one after the other, then the QR and the Jacobi of both at
+// once on the two half-warps, then ranks and splits one after the other.  The
+// same arithmetic per bond as two_site_update, in another lane arrangement (so
+// the same results up to the order of sums).
 template <int kD>
 __device__ __noinline__ void two_site_update_pair(const TrajParams& p, const Lay& Y, unsigned char* slot, int b1,
                                      const double2* G1, int b2, const double2* G2, bool adjoint, bool record,
@@ -881,8 +891,8 @@ static __device__ __noinline__ void order_layer(const TrajParams& p, const int* 
 // ---------------------------------------------------------------------------
 // Gradient of one layer (App. A), split so that each bond's gradient and its
 // costate update run back to back on one warp:
-//   layer_envs    left/right environments of <c|.|a> for the layer (warps 0
-//                 and 1) and the bonds ordered by cost (the last warp);
+//   layer_envs    left/right environments of <c|.|a> for the layer, by the even
+//                 and the odd warps;
 //   bond_gradient the mixed two-site density rho of bond b and dO/du =
 //                 tr(Q_u rho) for every control u of its gate, added to the
 //                 trajectory's gradient row as 2 Re(conj(O) dO/du); it leaves
@@ -1221,15 +1231,13 @@ __device__ __noinline__ void costate_group(const TrajParams& p, const Lay& Y, un
   }
 }
 
-// One layer of the costate sweep (App. A): the environments of <c_l|.|a_l>
-// (warps 0 and 1), then every bond of layer l -- largest first from the
-// shared counter -- its gradient and at once its costate update
+// One layer of the costate sweep (App. A): the environments of <c_l|.|a_l>,
+// then every bond of layer l -- largest first from the shared counter -- its
+// gradient and at once its costate update
 // c_{l-1} = G^dag c_l, which reuses the product c_b c_{b+1} the gradient
 // formed.  A bond's gradient reads only its own two costate sites and the
 // environments; its update rewrites those two sites, which no other bond of
-// the layer touches.  (Starting bonds while the environment sweeps still run
-// -- as soon as both are past the bond's sites -- measured slower: the sweeps
-// then share the FP64 pipes and the edge bonds wait for them all the same.)
+// the layer touches.
 template <int kD>
 __device__ void costate_layer(const TrajParams& p, const Lay& Y, unsigned char* cslot, const StateView av, int s,
                               int l, double2 wO, double* gsp_row, WarpCtx& w, int warp) {
