@@ -39,11 +39,20 @@ __device__ __forceinline__ double2 shfl4(double2 v, int src) {   // from lane sr
   return make_double2(__shfl_sync(0xffffffffu, v.x, src, 4), __shfl_sync(0xffffffffu, v.y, src, 4));
 }
 
+// 1 / sqrt(x) for x of normal FP32 size: the FP32 estimate (2e-7) and one
+// third-order step, seven FP64 instructions in the place of thirty.
+__device__ __forceinline__ double rsqrt_of(double x) {
+  const double y = (double)rsqrtf((float)x);
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
 // Cyclic Jacobi of the Hermitian 4 x 4 matrix whose row r is h: on return the
 // diagonal holds the eigenvalues and v is row r of V, h = V diag V^dagger.  A
-// round rotates two disjoint pairs (p, q), U = [[c, s], [-conj(s), c]]; the
-// angle is FP32 (each round still shrinks its off-diagonal entries by 1e-7),
-// the rotation unitary to FP64 rounding.  Returns false if it did not converge.
+// round rotates two disjoint pairs (p, q), U = [[c, s], [-conj(s), c]].  (Angles
+// from FP32, as in svd_fx.cuh, take a sweep more here: one fidelity of six
+// qubits 636 us against 619, 8 qubits with gradient 3.93 ms against 3.84, and
+// errors the same or a little larger.)  Returns false if it did not converge.
 __device__ bool herm_eig4_rows(double2 (&h)[4], double2 (&v)[4], int r) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) v[c] = make_double2(c == r ? 1.0 : 0.0, 0.0);
@@ -52,7 +61,7 @@ __device__ bool herm_eig4_rows(double2 (&h)[4], double2 (&v)[4], int r) {
   for (int c = 0; c < 4; ++c) sc += cabs2(h[c]);
   sc += __shfl_xor_sync(0xffffffffu, sc, 1, 4);
   sc += __shfl_xor_sync(0xffffffffu, sc, 2, 4);
-  // 2^-e with 2^(2e) about sc: the FP32 angles see entries of order one
+  // 2^-e with 2^(2e) about sc: angles from entries of order one
   const int e2 = (__double2hiint(sc) >> 20) & 2047;
   const double inv = __hiloint2double((1023 - ((e2 - 1023) >> 1)) << 20, 0);
   bool ok = false;
@@ -81,24 +90,20 @@ __device__ bool herm_eig4_rows(double2 (&h)[4], double2 (&v)[4], int r) {
       if (r == 0) hd = h[0];
       const double other = __shfl_sync(0xffffffffu, hd.x, mate, 4);
       const double2 z = shfl4(hm, low ? r : mate);
-      const float zx = (float)(z.x * inv), zy = (float)(z.y * inv);
-      const float z2 = fmaf(zx, zx, zy * zy);
-      float tx = 0.0f, ty = 0.0f;
-      if (z2 > 0.0f) {
-        const float d = (float)((low ? other - hd.x : hd.x - other) * inv);
-        const float iz = rsqrtf(z2), az = z2 * iz;
-        // tan = 2 |z| / (|d| + sqrt(d^2 + 4 |z|^2)), phase of z, sign of d
-        const float t = copysignf(2.0f * az * __fdividef(1.0f, fabsf(d) + sqrtf(fmaf(d, d, 4.0f * z2))), d);
-        tx = t * iz * zx;
-        ty = t * iz * zy;
+      const double zx = z.x * inv, zy = z.y * inv, d = (low ? other - hd.x : hd.x - other) * inv;
+      const double z2 = fma(zx, zx, zy * zy);
+      // with w = 1 / sqrt(d^2 + 4 |z|^2): cos 2theta = |d| w, c = sqrt((1 + cos
+      // 2theta) / 2), s = sign(d) w / c z
+      double c = 1.0;
+      double2 s = make_double2(0.0, 0.0);
+      if (z2 > 1e-35) {
+        const double w = rsqrt_of(fma(d, d, 4.0 * z2));
+        const double hq = fma(0.5, fabs(d) * w, 0.5);
+        const double rc = rsqrt_of(hq);
+        c = hq * rc;
+        const double f = copysign(w * rc, d);
+        s = make_double2(f * zx, f * zy);
       }
-      // c = 1 / sqrt(1 + |t|^2) by one third-order step from FP32, s = c t
-      const double dx = tx, dy = ty;
-      const double w = fma(dx, dx, fma(dy, dy, 1.0));
-      const double y0 = (double)rsqrtf((float)w);
-      const double e = fma(-w * y0, y0, 1.0);
-      const double c = fma(y0 * e, fma(e, 0.375, 0.5), y0);
-      const double2 s = make_double2(c * dx, c * dy);
       // columns of both pairs: (p, q) <- (c p - conj(s) q, s p + c q)
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
@@ -126,12 +131,9 @@ __device__ bool herm_eig4_rows(double2 (&h)[4], double2 (&v)[4], int r) {
         cfma(nh, sr, o);
         h[k] = nh;
       }
-      // an entry of 1e-10 is zero now up to 1e-17 (the FP32 angle) and rounding
-      if (z2 <= 1e-20f) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (k == mate) h[k] = make_double2(0.0, 0.0);
-      }
+      for (int k = 0; k < 4; ++k)
+        if (k == mate) h[k] = make_double2(0.0, 0.0);
     }
   }
   return ok;
