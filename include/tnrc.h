@@ -99,7 +99,9 @@ typedef struct {
   int32_t ctas_per_sm;           /* resident trajectory CTAs per SM, 1..4, clamped to
                                     warps_per_cta * ctas_per_sm <= 16; above 8 warps per SM
                                     the kernel's 128-register build runs; 0 = 1, or 2 CTAs of
-                                    4 warps when both are 0 and the trajectories fill them  */
+                                    4 warps when both are 0, the trajectories fill them, their
+                                    work regions take at most 32 GiB and (operators) half of
+                                    an SM's shared memory holds the largest theta           */
   int32_t crosstalk_terms;       /* 1 (or 0): J^z ZZ per bond, J[M][N-1]; 3: the Heisenberg
                                     type J^x XX + J^y YY + J^z ZZ of Eq. Hp, J[M][N-1][3]
                                     in the order (x, y, z)                                 */
@@ -135,8 +137,7 @@ typedef struct {
                                     did not fit their CTA's region packed and that were redone
                                     with checkpoints (results are identical either way)     */
   int64_t phase_cycles[9];       /* SM cycles summed over warps per phase of the trajectory
-                                    kernel (contraction, pivoted QR and the second QR,
-                                    rank/truncate, split, environments, gradients, history
+                                    kernel (contraction, pivoted QR, rank/truncate, split, environments, gradients, history
                                     copies, layer barriers, Jacobi sweeps); zero unless
                                     built with TNRC_PHASE_TIMERS                            */
   int64_t cap_truncations;       /* truncations of the last evaluation (forward and costate
@@ -224,14 +225,15 @@ tnrc_status tnrc_set_graphs(tnrc_ctx* ctx, int32_t enable);
  * tnrc_fidelity_grad, and TNRC_E_NOMEM. */
 tnrc_status tnrc_fidelity_grad_plain(tnrc_ctx* ctx, double* F, double* grad);
 
-/* Matrix shape of the trajectory kernel's SVDs: pairs = 1 (the default) lets
- * a warp take two small two-site updates at once, their pivoted QR and
- * Jacobi SVDs running on the two half-warps (when both thetas and both Phis
- * fit the warp's shared slab and no side exceeds 64), so the per-round
- * scalar work of the Jacobi is shared by two matrices; pairs = 0 gives every
- * SVD a whole warp.  Results agree within rounding (the sums run in another
- * lane arrangement); the plain path follows the same setting.  Captured
- * graphs are dropped when it changes.  The autotuner picks it per shape. */
+/* Matrix shape of the trajectory kernel's SVDs on chains of 33 sites or more:
+ * pairs = 1 (the default) lets a warp take two small two-site updates at once,
+ * their pivoted QR and Jacobi SVDs running on the two half-warps (when both
+ * fit the warp's shared slab and no side exceeds 64), so the per-round scalar
+ * work of the Jacobi is shared by two matrices; pairs = 0 gives every SVD a
+ * whole warp.  (On shorter chains a warp takes one bond at a time, and a large
+ * update is shared by all warps of the CTA, in either setting.)  Results agree
+ * within rounding; the plain path follows the same setting.  Captured graphs
+ * are dropped when it changes.  The autotuner picks it per shape. */
 tnrc_status tnrc_set_svd_shape(tnrc_ctx* ctx, int32_t pairs);
 
 /* Order the context's later work on another stream (a cudaStream_t; NULL =

@@ -134,9 +134,22 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
   // two CTAs of half the warps once the trajectories fill them: each CTA's
   // serial stretches (environment sweeps, layer barriers) then run beside the
   // other's updates (cnot50 near the solution, 304 trajectories: 479 ms as 8
-  // x 1, 386 ms as 4 x 2; with 152 trajectories of ghz30, 172 and 233 ms)
-  const bool two = pb->warps_per_cta == 0 && pb->ctas_per_sm == 0 && P.warps == tnrc::kWarps &&
-                   2 * T >= 3ll * n_sm;
+  // x 1, 386 ms as 4 x 2; with 152 trajectories of ghz30, 172 and 233 ms).
+  // Not where the second set of work regions would take tens of GB: a default
+  // leaves room for other contexts (a caller can still ask for it).
+  // Nor for operators whose largest theta and R^dagger leave half of an SM's
+  // shared memory: their bonds do reach the cap, and the CTA then works on them
+  // in global scratch (chi 16, 300 trajectories: 4 sites 16.5 ms as 8 x 1 and
+  // 12.5 as 4 x 2, 8 sites 379 and 657; 5 sites, 600 trajectories: 77 and 59).
+  bool two = pb->warps_per_cta == 0 && pb->ctas_per_sm == 0 && 2 * T >= 3ll * n_sm &&
+             2ll * n_sm * (2 + P.nseg + P.seg) * P.L.bytes <= (32ll << 30);
+  if (two && P.d == 4) {
+    const long long half = (110 * 1024 - (int)tnrc_traj_smem(tnrc::kWarps / 2, 0) - 1024) / 16;
+    for (int b = 0; b + 2 <= N; ++b) {
+      const long long m = 4ll * P.dcap[b], n = 4ll * P.dcap[b + 2];
+      two = two && m * n + std::min(m, n) * (n | 1) + m <= half;
+    }
+  }
   if (two) P.warps = tnrc::kWarps / 2;
   if (pb->warps_per_cta > 0) P.warps = pb->warps_per_cta;
   if (const char* e = getenv("TNRC_WARPS")) {
