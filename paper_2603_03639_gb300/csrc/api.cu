@@ -133,8 +133,6 @@ tnrc::TrajParams traj_params(tnrc_ctx* ctx, bool grad) {
   tp.warp_scratch = ctx->at<double2>(P.off_scratch);
   tp.scratch_elems = P.scratch_elems;
   tp.env_scratch = ctx->at<double2>(P.off_env);
-  tp.env_elems = P.env_elems;
-  tp.site_elems = P.site_elems;
   tp.lgates = ctx->at<tnrc::LayerGate>(P.off_gates);
   tp.layer_off = ctx->at<int>(P.off_loff);
   tp.n_layers = P.n_layers;

@@ -118,11 +118,13 @@ template <int kD>
 __global__ void __launch_bounds__(64) plain_envs_kernel(TrajParams p, const unsigned char* cslot,
                                                         const unsigned char* aslot) {
   __shared__ int s_order[1], s_next;
-  __shared__ WideShared s_wide;
   WarpCtx w;
   const int warp = threadIdx.x >> 5;
-  plain_warp(p, w, warp, s_order, &s_next, warp, &s_wide);
-  layer_to_fx<kD>(p, p.full, cslot, slot_view(aslot, p.full), w);
+  plain_warp(p, w, warp, s_order, &s_next, warp);
+  if (threadIdx.x == 0) {
+    env_left(p, w.region)[0] = make_double2(1.0, 0.0);
+    env_right(p, w.region)[(size_t)p.N * p.chi * p.chi] = make_double2(1.0, 0.0);
+  }
   __syncthreads();
   layer_envs<kD>(p, p.full, cslot, slot_view(aslot, p.full), w, warp);
 }

@@ -71,7 +71,6 @@ struct Plan {
   int64_t scratch_elems;      // per warp
   int64_t work_stride;        // bytes per CTA
   int64_t env_elems;          // per CTA
-  int64_t site_elems;         // complex elements of a slot's site tensors
   // arena offsets (bytes)
   int64_t off_loff;
   int64_t off_u, off_mask, off_gfix, off_J, off_gates, off_in, off_tg, off_work, off_scratch, off_env, off_O,
@@ -171,12 +170,11 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
     P.slab_elems = std::max(256, std::min(P.d * P.d * chi * chi, per_warp / 32 * 32));
   }
   const int64_t cc = (int64_t)chi * chi;
-  // per warp: Phi (d chi)^2, theta (d chi)^2, then the gradient's four
-  // intermediates (at most (d + 3 d^2) chi^2) past 2 (d chi)^2
-  P.scratch_elems = (5 * (int64_t)P.d * P.d + P.d) * cc;
-  // left and right environments, both states' sites in integers, exponents
-  P.site_elems = (P.L.bytes - P.L.sites_off) / 16;
-  P.env_elems = 2 * (int64_t)(N + 1) * cc + 2 * P.site_elems + (N + 2);
+  // per warp: Phi (d chi)^2, theta (d chi)^2, then the gradient's three
+  // intermediates (at most (d + 2 d^2) chi^2) or the R^dagger of a wide update
+  // past 2 (d chi)^2
+  P.scratch_elems = (4 * (int64_t)P.d * P.d + P.d) * cc;
+  P.env_elems = 2 * (int64_t)(N + 1) * cc;
   P.work_stride = (int64_t)(2 + P.nseg + P.seg) * P.L.bytes;
   const int64_t per_cta = P.work_stride + (P.scratch_elems * P.warps + P.env_elems) * 16;
   int grid = (int)std::min<long long>(T, (long long)n_sm * ctas_per_sm);

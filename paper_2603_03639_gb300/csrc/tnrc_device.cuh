@@ -110,9 +110,7 @@ struct TrajParams {
   int64_t work_stride;             // bytes per CTA
   double2* warp_scratch;           // per warp: scratch_elems complex
   int64_t scratch_elems;
-  double2* env_scratch;            // per CTA: env_elems complex (EnvMem in traj_impl.cuh)
-  int64_t env_elems;
-  int64_t site_elems;              // complex elements of a slot's site tensors
+  double2* env_scratch;            // per CTA: 2*(N+1)*chi*chi complex
   const LayerGate* lgates;         // [M][recs_per_sample]: layer l's bonds at layer_off[l]
   const int* layer_off;            // [n_layers + 1]
   int n_layers;                    // truncated layers of one trajectory

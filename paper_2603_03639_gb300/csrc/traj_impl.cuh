@@ -23,9 +23,9 @@
 // Each trajectory writes its own O and its own gradient row, so results do not
 // depend on which CTA ran it or on what else ran in the launch.
 //
-// What bounds it: with the SVDs, the environments and the gradients in integers
-// (fx.cuh) the FP64 pipe is 13 % busy on the 50-qubit benchmark and DRAM at 1 %;
-// a warp waits for the results of its own instructions (fixed latencies a third
+// What bounds it: with the SVDs in integers (fx.cuh) neither the FP64 pipe nor
+// DRAM is busy for long (profiles/traj_kernel_cnot50_counters.txt); a warp waits
+// for the results of its own instructions (fixed latencies a third
 // of the stalls, then shared and L2 loads, barriers and instruction fetch), two
 // warps to a scheduler, which the 220 KB of shared memory for theta and
 // R^dagger allow.  Every function is out of line and no runtime loop unrolled:
@@ -72,7 +72,6 @@ struct WideShared {
   double part[kWarps];
   FxQrShared qr;
   long long total;   // cost of the current layer
-  int ring[6];       // largest entries of the environment steps
   int k;
 };
 
@@ -656,161 +655,64 @@ __device__ __noinline__ size_t pack_state(const TrajParams& p, const Lay& Y, con
 }
 
 // ---------------------------------------------------------------------------
-// Transfer-matrix steps of <c| . |a>.
+// Transfer-matrix steps of <c| . |a>, in FP64.  (In 56-bit integers with one scale
+// per tensor the gradient cases were 2 to 7 % faster, but sums of dense operators
+// left the range and overlaps of weak controls lost their digits: an environment
+// spans as many decades as the overlap does.)
 // Left:  Eout[b'][a'] = sum_{b,s,a} conj(c[b][s][b']) Ein[b][a] a[a][s][a']
 // Right: Eout[b][a]   = sum_{s,b',a'} conj(c[b][s][b']) Ein[b'][a'] a[a][s][a']
 // ---------------------------------------------------------------------------
 
-// The left step of the final overlap, by one warp in FP64.
-template <int kD>
-__device__ __noinline__ void overlap_step(const double2* Ein, int Dcl, int Dal, const double2* c, int Dcr,
-                                          const double2* a, int Dar, double2* tmp, double2* Eout, int ti) {
-  const int nt = 32;
-  const int w2 = kD * Dar;
-#pragma unroll 1
-  for (int it = ti; it < Dcl * w2; it += nt) {
-    const int be = it / w2, rest = it - be * w2;
-    double2 acc = make_double2(0.0, 0.0);
-#pragma unroll 1
-    for (int al = 0; al < Dal; ++al) cfma(acc, Ein[be * Dal + al], a[(size_t)al * w2 + rest]);
-    tmp[it] = acc;
-  }
-  __syncwarp();
-#pragma unroll 1
-  for (int it = ti; it < Dcr * Dar; it += nt) {
-    const int bp = it / Dar, ap = it - bp * Dar;
-    double2 acc = make_double2(0.0, 0.0);
-#pragma unroll 1
-    for (int be = 0; be < Dcl; ++be)
-#pragma unroll
-      for (int s = 0; s < kD; ++s)
-        cfmac(acc, c[(size_t)be * kD * Dcr + s * Dcr + bp], tmp[(size_t)be * w2 + s * Dar + ap]);
-    Eout[it] = acc;
-  }
-  __syncwarp();
+// Environments of a region: chi^2 elements per bond, L_0 .. L_N and R_0 .. R_N.
+__device__ __forceinline__ double2* env_left(const TrajParams& p, int region) {
+  return p.env_scratch + (size_t)region * 2 * (p.N + 1) * p.chi * p.chi;
+}
+__device__ __forceinline__ double2* env_right(const TrajParams& p, int region) {
+  return env_left(p, region) + (size_t)(p.N + 1) * p.chi * p.chi;
 }
 
-// ---------------------------------------------------------------------------
-// The environments and the gate gradients of the costate sweep in fixed point.
-// They are sums over whole bonds that only the gradient reads, so one scale per
-// tensor keeps all that it needs (what the updates read stays FP64).  Every site
-// tensor of the two states is brought to integers once per layer, its largest
-// entry near 2^55; an environment carries the exponent of its own largest entry.
-// In FP64 (a complex multiply-add is four instructions of 64 cycles, in integers
-// twelve of five) these two took a third of a small evaluation.
-// ---------------------------------------------------------------------------
-struct EnvMem {
-  int4 *L, *R;       // environments, chi^2 elements per bond
-  int4 *c, *a;       // site tensors of the costate and of the forward state, at slot offsets
-  int *eL, *eR;      // exponents of the environments [N+1], real value = v 2^(e - 55)
-  int *ec, *ea;      // exponents of the site tensors [N]
-};
-__device__ __forceinline__ EnvMem env_mem(const TrajParams& p, int region) {
-  const size_t cc = (size_t)p.chi * p.chi, ne = (size_t)(p.N + 1) * cc;
-  EnvMem m;
-  m.L = reinterpret_cast<int4*>(p.env_scratch + (size_t)region * p.env_elems);
-  m.R = m.L + ne;
-  m.c = m.R + ne;
-  m.a = m.c + p.site_elems;
-  m.eL = reinterpret_cast<int*>(m.a + p.site_elems);
-  m.eR = m.eL + p.N + 1;
-  m.ec = m.eR + p.N + 1;
-  m.ea = m.ec + p.N + 1;
-  return m;
-}
-
-// Sum of products / 2^55 2^sh, |sh| <= 26.
-__device__ __forceinline__ long long fx_sum55(FxAcc s, int sh) {
-  const long long h = sh >= -1 ? s.h << (1 + sh) : s.h >> (-1 - sh);
-  return h + ((s.x + (1ll << (26 - sh))) >> (27 - sh));
-}
-
-// A site tensor (cnt entries) to integers, by one warp.
-static __device__ __noinline__ void site_to_fx(const double2* src, int cnt, int4* dst, int* ex, int lane) {
-  int mx = 0;
-#pragma unroll 1
-  for (int e = lane; e < cnt; e += 32) {
-    const double2 v = src[e];
-    mx = max(mx, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
-  }
-  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
-  const int x = (mx >> 20) - 1022;
-#pragma unroll 1
-  for (int e = lane; e < cnt; e += 32) dst[e] = fx_from_double2(src[e], 55 - x);
-  if (lane == 0) *ex = x;
-}
-
-// Every thread of the CTA: both states' sites, and the outermost environments.
-template <int kD>
-__device__ __noinline__ void layer_to_fx(const TrajParams& p, const Lay& Y, const unsigned char* cslot,
-                                         const StateView av, WarpCtx& w) {
-  const EnvMem m = env_mem(p, w.region);
-  const int* Dc = slot_dims(cslot);
-  const double2* cs = slot_sites(cslot, Y.L);
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll 1
-  for (int u = warp; u < 2 * p.N; u += nw) {
-    const int i = u >> 1, off = Y.site_off[i];
-    if (u & 1)
-      site_to_fx(av.sites + av.off[i], av.D[i] * kD * av.D[i + 1], m.a + off, m.ea + i, w.lane);
-    else
-      site_to_fx(cs + off, Dc[i] * kD * Dc[i + 1], m.c + off, m.ec + i, w.lane);
-  }
-  if (threadIdx.x == 0) {
-    const int4 one = make_int4(1 << 27, 0, 0, 0);
-    m.L[0] = one;
-    m.R[(size_t)p.N * p.chi * p.chi] = one;
-    m.eL[0] = 0;
-    m.eR[p.N] = 0;
-    for (int t = 0; t < 6; ++t) w.wide->ring[t] = 0;
-  }
-}
-
-// The team of one sweep meets at its named barrier.
+// The team of one sweep meets at its named barrier; a single warp (team < 0)
+// needs none.
 __device__ __forceinline__ void team_sync(int team, int nt) {
-  if (team == 0)
-    asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
+  if (team < 0)
+    __syncwarp();
   else
-    asm volatile("bar.sync 2, %0;" ::"r"(nt) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(nt) : "memory");
 }
 
-// One step by thread ti of nt.  The first product takes the shift sh that brings
-// the environment's largest entry to 2^55; the largest entry of the result (as
-// its bit length) is left in *bits.  Left (team 0): k runs over the left bonds.
+// One step by thread ti of nt, in FP64.  Left (team 0, or one warp with team -1):
+// k runs over the left bonds.  Every element is summed by one thread in a fixed
+// order, so results do not depend on the team.
 template <int kD>
-__device__ __noinline__ void env_step(int team, const int4* Ein, int D1, int K1, const int4* c, int cs1, int cs2,
-                                      const int4* a, int as1, int as2, int D2, int Da2, int4* tmp, int4* Eout, int sh,
-                                      int* bits, int ti, int nt) {
+__device__ __noinline__ void env_step(int team, const double2* Ein, int D1, int K1, const double2* c, int cs1, int cs2,
+                                      const double2* a, int as1, int as2, int D2, int Da2, double2* tmp, double2* Eout,
+                                      int ti, int nt) {
   // tmp[i][s][y] = sum_k Ein[i][k] a(k, s, y), i < D1, k < K1, y < Da2; a(k, s, y) at
   // k as1 + s Da' + y as2 (s stride: Da2 on the left, K1 on the right)
-  const int as_s = team == 0 ? Da2 : K1, w2 = kD * Da2;
+  const bool left = team != 1;
+  const int as_s = left ? Da2 : K1, w2 = kD * Da2;
 #pragma unroll 1
   for (int it = ti; it < D1 * w2; it += nt) {
     const int i = it / w2, rest = it - i * w2, s = rest / Da2, y = rest - s * Da2;
-    const int4* ap = a + s * as_s + y * as2;
-    FxAcc re{0, 0}, im{0, 0};
+    const double2* ap = a + s * as_s + y * as2;
+    double2 acc = make_double2(0.0, 0.0);
 #pragma unroll 2
-    for (int k = 0; k < K1; ++k) fx_cmac(re, im, Ein[i * K1 + k], ap[k * as1]);
-    tmp[it] = fx_pack(fx_sum55(re, sh), fx_sum55(im, sh));
+    for (int k = 0; k < K1; ++k) cfma(acc, Ein[i * K1 + k], ap[k * as1]);
+    tmp[it] = acc;
   }
   team_sync(team, nt);
   // Eout[x][y] = sum_{i,s} conj(c(i, s, x)) tmp[i][s][y], c(i, s, x) at i cs1 + s cs' + x cs2
-  const int cs_s = team == 0 ? D2 : D1;
-  long long top = 0;
+  const int cs_s = left ? D2 : D1;
 #pragma unroll 1
   for (int it = ti; it < D2 * Da2; it += nt) {
     const int x = it / Da2, y = it - x * Da2;
-    FxAcc re{0, 0}, im{0, 0};
+    double2 acc = make_double2(0.0, 0.0);
 #pragma unroll 1
     for (int i = 0; i < D1; ++i)
 #pragma unroll
-      for (int s = 0; s < kD; ++s) fx_cmacc(re, im, c[i * cs1 + s * cs_s + x * cs2], tmp[i * w2 + s * Da2 + y]);
-    const long long vr = fx_sum55(re, 0), vi = fx_sum55(im, 0);
-    top |= (vr < 0 ? -vr : vr) | (vi < 0 ? -vi : vi);
-    Eout[it] = fx_pack(vr, vi);
+      for (int s = 0; s < kD; ++s) cfmac(acc, c[i * cs1 + s * cs_s + x * cs2], tmp[i * w2 + s * Da2 + y]);
+    Eout[it] = acc;
   }
-  const int b = (int)__reduce_max_sync(0xffffffffu, (unsigned)(64 - __clzll(top)));
-  if ((threadIdx.x & 31) == 0) atomicMax(bits, b);
   team_sync(team, nt);
 }
 
@@ -830,8 +732,8 @@ __device__ __noinline__ double2 warp_overlap(const TrajParams& p, const Lay& Yt,
   __syncwarp();
 #pragma unroll 1
   for (int i = 0; i < p.N; ++i) {
-    overlap_step<kD>(E0, Dt[i], Da[i], ts + Yt.site_off[i], Dt[i + 1], as + Ya.site_off[i], Da[i + 1], tmp, E1,
-                     w.lane);
+    env_step<kD>(-1, E0, Dt[i], Da[i], ts + Yt.site_off[i], kD * Dt[i + 1], 1, as + Ya.site_off[i], kD * Da[i + 1], 1,
+                 Dt[i + 1], Da[i + 1], tmp, E1, w.lane, 32);
     double2* x = E0;
     E0 = E1;
     E1 = x;
@@ -907,59 +809,47 @@ __device__ __noinline__ void layer_envs(const TrajParams& p, const Lay& Y, const
   const size_t cc = (size_t)p.chi * p.chi;
   const int* Dc = slot_dims(cslot);
   const int* Da = av.D;
-  const int* off = Y.site_off;
-  const EnvMem m = env_mem(p, w.region);
+  const double2* cs = slot_sites(cslot, Y.L);
+  double2* L = env_left(p, w.region);
+  double2* R = env_right(p, w.region);
 
   // left environments L_i (sites < i) for i <= N-2 by the even warps, right
   // R_i (sites >= i) for i >= 2 by the odd warps: each sweep is sequential
   // over the sites, so each step is shared by its team of warps; the step's
   // intermediate (at most Dc x kD Da) sits in the team's first warp's shared
-  // slab when it fits, else in its scratch.  Each element is summed by one
-  // thread, so the result does not depend on the team.
+  // slab when it fits, else in its scratch.
   TNRC_TIC(t_e);
   const int team = warp & 1;                               // 0: left, 1: right
   const int nt = 32 * (team == 0 ? (p.warps + 1) / 2 : p.warps / 2);
   const int ti = (warp >> 1) * 32 + w.lane;
-  int4* lead_slab = reinterpret_cast<int4*>(w.slab - (size_t)(warp - team) * p.slab_elems);
-  int4* lead_scratch = reinterpret_cast<int4*>(w.scratch - (size_t)(warp - team) * p.scratch_elems);
-  int* ring = w.wide->ring + 3 * team;   // largest entries of three steps in turn
-  int sh = 0, e = 0;
+  double2* lead_slab = w.slab - (size_t)(warp - team) * p.slab_elems;
+  double2* lead_scratch = w.scratch - (size_t)(warp - team) * p.scratch_elems;
 #pragma unroll 1
   for (int t = 0; t < N - 2; ++t) {
     const int i = team == 0 ? t : N - 1 - t;               // the site taken in
-    int* bits = ring + t % 3;
     const int cl = Dc[i], cr = Dc[i + 1], al = Da[i], ar = Da[i + 1];
     const int n1 = kD * (team == 0 ? cl * ar : cr * al);
-    int4* tmp = n1 <= p.slab_elems ? lead_slab : lead_scratch;
-    const int4 *c = m.c + off[i], *a = m.a + off[i];
+    double2* tmp = n1 <= p.slab_elems ? lead_slab : lead_scratch;
+    const double2 *c = cs + Y.site_off[i], *a = av.sites + av.off[i];
     if (team == 0)
-      env_step<kD>(0, m.L + i * cc, cl, al, c, kD * cr, 1, a, kD * ar, 1, cr, ar, tmp, m.L + (i + 1) * cc, sh, bits, ti,
-                   nt);
+      env_step<kD>(0, L + i * cc, cl, al, c, kD * cr, 1, a, kD * ar, 1, cr, ar, tmp, L + (i + 1) * cc, ti, nt);
     else
-      env_step<kD>(1, m.R + (i + 1) * cc, cr, ar, c, 1, kD * cr, a, 1, kD * ar, cl, al, tmp, m.R + i * cc, sh, bits, ti,
-                   nt);
-    e += m.ec[i] + m.ea[i] - sh;
-    const int b = *bits;
-    sh = b > 0 ? max(-26, min(26, 55 - b)) : 0;
-    if (ti == 0) {
-      (team == 0 ? m.eL : m.eR)[team == 0 ? i + 1 : i] = e;
-      ring[(t + 2) % 3] = 0;   // read by every thread before the barrier within this step
-    }
+      env_step<kD>(1, R + (i + 1) * cc, cr, ar, c, 1, kD * cr, a, 1, kD * ar, cl, al, tmp, R + i * cc, ti, nt);
     if (ti == 0) w.alg += 8ull * n1 * (unsigned long long)(team == 0 ? al : ar) + 8ull * kD * cl * cr * (team == 0 ? ar : al);
   }
   TNRC_TOC(w, 4, t_e);
 }
 
 // out[i][j] = sum_k A[i K + k] B(k, j), M x J outputs, B(k, j) at k bk + j bj.
-static __device__ __noinline__ void fx_gemm(const int4* A, const int4* B, int M, int K, int J, int bk, int bj, int4* out,
-                                            int ti, int nt) {
+static __device__ __noinline__ void small_gemm(const double2* A, const double2* B, int M, int K, int J, int bk, int bj,
+                                               double2* out, int ti, int nt) {
 #pragma unroll 1
   for (int it = ti; it < M * J; it += nt) {
     const int i = it / J, j = it - i * J;
-    FxAcc re{0, 0}, im{0, 0};
+    double2 acc = make_double2(0.0, 0.0);
 #pragma unroll 2
-    for (int k = 0; k < K; ++k) fx_cmac(re, im, A[i * K + k], B[k * bk + j * bj]);
-    out[it] = fx_pack(fx_sum55(re, 0), fx_sum55(im, 0));
+    for (int k = 0; k < K; ++k) cfma(acc, A[i * K + k], B[k * bk + j * bj]);
+    out[it] = acc;
   }
 }
 
@@ -973,7 +863,10 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
   const int* Da = av.D;
   const double2* cs = slot_sites(cslot, Y.L);
   const int* so = Y.site_off;
-  const EnvMem em = env_mem(p, w.region);
+  const double2* L = env_left(p, w.region) + (size_t)b * cc;
+  const double2* R = env_right(p, w.region) + (size_t)(b + 2) * cc;
+  const double2* a0 = av.sites + av.off[b];
+  const double2* a1 = av.sites + av.off[b + 1];
   const int lane = w.lane;
   const int ti = cta ? (int)threadIdx.x : lane, nt = cta ? (int)blockDim.x : 32;
   auto sync = [&]() {
@@ -992,22 +885,19 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
   if (ti < 32)
     w.alg += 8ull * dcl * (kD * dam * dal + kDD * dar * dam + kDD * dcr * dar +
                            (unsigned long long)kDD * kDD * dcr) + 2048ull;
-  // Wc = c_b c_{b+1} [dcl][kD^2][dcr] at Wc (theta's home), in FP64 for the update
-  // that takes it over; the integer intermediates packed at their actual sizes
-  // right after it in the shared slab when they fit there, else in global
-  // scratch past theta's room
+  // Wc = c_b c_{b+1} [dcl][kD^2][dcr] at Wc (theta's home); the other three
+  // intermediates packed at their actual sizes right after it in the shared
+  // slab when they fit there, else in global scratch past theta's room
   const int n1 = dcl * kD * dam, n2 = dcl * kDD * dar, n3 = dcl * kDD * dcr;
   double2* slab = cta ? w.cta_slab : w.slab;
   const int slab_elems = cta ? p.cta_slab_elems : p.slab_elems;
   const bool wc_in_slab = Wc >= slab && Wc < slab + slab_elems;
-  int4* U1 = reinterpret_cast<int4*>((wc_in_slab && (Wc - slab) + n3 + n1 + n2 + 2 * n3 <= slab_elems)
-                                         ? Wc + n3
-                                         : (cta ? w.cta_scratch : w.scratch) + (size_t)2 * kDD * chi * chi);
-  int4* U2 = U1 + n1;   // U1 [dcl][kD][dam], U2 [dcl][kD^2][dar]
-  int4* U3 = U2 + n2;   // [dcl][kD^2][dcr]
-  int4* Wi = U3 + n3;   // Wc in integers
-  const int ew = em.ec[b] + em.ec[b + 1] + 2;   // |Wc| < 2^ew with room to spare
-  fx_gemm(em.L + (size_t)b * cc, em.a + so[b], dcl, dal, kD * dam, kD * dam, 1, U1, ti, nt);
+  double2* U1 = (wc_in_slab && (Wc - slab) + n3 + n1 + n2 + n3 <= slab_elems)
+                    ? Wc + n3
+                    : (cta ? w.cta_scratch : w.scratch) + (size_t)2 * kDD * chi * chi;
+  double2* U2 = U1 + n1;   // U1 [dcl][kD][dam], U2 [dcl][kD^2][dar]
+  double2* U3 = U2 + n2;   // [dcl][kD^2][dcr]
+  small_gemm(L, a0, dcl, dal, kD * dam, kD * dam, 1, U1, ti, nt);
 #pragma unroll 1
   for (int it = ti; it < dcl * kDD * dcr; it += nt) {
     const int be = it / (kDD * dcr), rest = it - be * kDD * dcr;
@@ -1018,12 +908,11 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
     for (int b1 = 0; b1 < dcm; ++b1)
       cfma(acc, c0[(size_t)be * kD * dcm + s1 * dcm + b1], c1[(size_t)b1 * kD * dcr + s2 * dcr + b2]);
     Wc[it] = acc;
-    Wi[it] = fx_from_double2(acc, 55 - ew);
   }
   sync();
-  fx_gemm(U1, em.a + so[b + 1], dcl * kD, dam, kD * dar, kD * dar, 1, U2, ti, nt);
+  small_gemm(U1, a1, dcl * kD, dam, kD * dar, kD * dar, 1, U2, ti, nt);
   sync();
-  fx_gemm(U2, em.R + (size_t)(b + 2) * cc, dcl * kDD, dar, dcr, 1, dar, U3, ti, nt);
+  small_gemm(U2, R, dcl * kDD, dar, dcr, 1, dar, U3, ti, nt);
   sync();
   // rho[o'][o] = sum_{i1,i2} sum_{be,b2} U3[be][s'][b2] conj(Wc[be][s][b2]) over the
   // two-site out indices o (the in indices, if any, traced out: the gate acts
@@ -1033,12 +922,11 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
   {
     const int parts = cta ? 8 : 2;
     double2* sums = cta ? w.cta_small : w.small;   // at least two warps' 64 elements
-    const int e = em.eL[b] + em.ea[b] + em.ea[b + 1] + em.eR[b + 2] + ew;
 #pragma unroll 1
     for (int it = ti; it < 16 * parts; it += nt) {
       const int o = it & 15, part = it >> 4;
       const int op = o >> 2, oq = o & 3;
-      FxAcc re{0, 0}, im{0, 0};
+      double2 acc = make_double2(0.0, 0.0);
 #pragma unroll 1
       for (int ii = 0; ii < kI * kI; ++ii) {
         const int i1 = ii / kI, i2 = ii % kI;
@@ -1046,13 +934,13 @@ __device__ __noinline__ void bond_gradient(const TrajParams& p, const Lay& Y, co
         const int sq = ((oq >> 1) * kI + i1) * kD + (oq & 1) * kI + i2;
 #pragma unroll 1
         for (int be = part; be < dcl; be += parts) {
-          const int4* u = U3 + (size_t)be * kDD * dcr + sp * dcr;
-          const int4* wv = Wi + (size_t)be * kDD * dcr + sq * dcr;
+          const double2* u = U3 + (size_t)be * kDD * dcr + sp * dcr;
+          const double2* wv = Wc + (size_t)be * kDD * dcr + sq * dcr;
 #pragma unroll 1
-          for (int b2 = 0; b2 < dcr; ++b2) fx_cmacc(re, im, wv[b2], u[b2]);
+          for (int b2 = 0; b2 < dcr; ++b2) cfmac(acc, wv[b2], u[b2]);
         }
       }
-      sums[it] = make_double2(fx_scale((double)fx_sum55(re, 0), e - 55), fx_scale((double)fx_sum55(im, 0), e - 55));
+      sums[it] = acc;
     }
     sync();
     if (ti < 16) {
@@ -1246,7 +1134,10 @@ __device__ void costate_layer(const TrajParams& p, const Lay& Y, unsigned char* 
   const int lane = w.lane;
   const int* Dc = slot_dims(cslot);
   if (warp == p.warps - 1) order_layer(p, Dc, parity, w);
-  layer_to_fx<kD>(p, Y, cslot, av, w);
+  if (threadIdx.x == 0) {
+    env_left(p, w.region)[0] = make_double2(1.0, 0.0);
+    env_right(p, w.region)[(size_t)p.N * p.chi * p.chi] = make_double2(1.0, 0.0);
+  }
   __syncthreads();
   layer_envs<kD>(p, Y, cslot, av, w, warp);
   __syncthreads();
