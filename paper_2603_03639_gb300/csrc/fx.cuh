@@ -122,6 +122,27 @@ TNRC_HD float fx_to_float(long long v) {
   return (float)hi * 4294967296.0f + (float)lo;
 }
 
+// Entries of a Gram-Schmidt row, by the bits of their high limbs: a row is taken
+// down by 2^fx_row_shift (to below 2^54) once an entry has passed 2^55.  An update
+// c -= p (r y), |r y| <= 1, at most doubles an entry (2.5 times by components), so
+// entries stay below 2^57, a quarter of what two limbs hold.
+TNRC_HD int fx_high_bits(int hi) { return hi ^ (hi >> 31); }
+TNRC_HD int fx_row_shift(int high_bits) {
+  int k = 0;
+  if (high_bits >= (1 << 27))
+    while ((high_bits >> k) >= (1 << 26)) ++k;
+  return k;
+}
+
+// The exponent kw of a pivot column's weighted copy, p_i 2^(2 er_i + kw): entries
+// below 2^54 (top: the largest log2 |p_i 2^(2 er_i)|^2), and inner products with the
+// remaining columns, which |p|^2 2^kw bounds (pn = |p|^2, the largest left), below
+// 2^(56 + 58).
+TNRC_HD int fx_pivot_weight(int top, float pn) {
+  const int a = (107 - top) >> 1, b = 113 - fx_ilog2f(pn);
+  return a < b ? a : b;
+}
+
 // 1 / sqrt(N 2^-56) in units of 2^-56, for N in about [2^54, 2^56]: the float
 // estimate y0 and one third-order step, y = y0 (1 + e/2 + 3 e^2 / 8) with e =
 // 1 - a y0^2 formed in integers.

@@ -131,10 +131,11 @@ __device__ __forceinline__ int fx_umax(int v) { return (int)__reduce_max_sync(0x
 // theta's rows are graded (row (al, s) carries the Schmidt value lam_al, down
 // to 1e-12 of the largest), and the small singular vectors live in the small
 // rows, so every row has a scale of its own: theta = W 2^(er[row] + E0), the
-// largest entry of a row near 2^54 and er <= 0.  (One scale for the whole
-// matrix loses the digits of components of weight 1e-6, which an overlap of
-// 1e-7 still depends on.)  Inner products over rows use a weighted copy of the
-// pivot column, Pw = p 2^(2 er + kw); the update of a column needs no weights.
+// largest entry of a row near 2^54 and kept below 2^55 (fx_rescale_rows).  (One
+// scale for the whole matrix loses the digits of components of weight 1e-6, which
+// an overlap of 1e-7 still depends on.)  Inner products over rows use a weighted
+// copy of the pivot column, Pw = p 2^(2 er + kw); the update of a column needs no
+// weights.
 //
 // thr: squared norm (in units of 2^(2 E0)) at which the remaining columns count
 // as zero.  Column j of R^dagger goes to X + j ldx (n entries) with exponent
@@ -222,10 +223,11 @@ __device__ __forceinline__ unsigned fx_pivot_key(const float* cn, const int* ord
 }
 
 // Pivot column p by lw lanes: its squared norm 2^-56 at full scale (entries
-// p 2^(er + k)), and the weighted copy Pw = p 2^(2 er + kw), |Pw| < 2^55.
+// p 2^(er + k)), and the weighted copy Pw = p 2^(2 er + kw).  pn: the squared norm
+// in FP32.
 template <bool SH>
-__device__ __forceinline__ long long fx_pivot(const FxMem<SH>& W, int4* Pw, int m, int n, int p, int k, const int* er,
-                                              bool on, int ll, int lw, int& kw) {
+__device__ __forceinline__ long long fx_pivot(const FxMem<SH>& W, int4* Pw, int m, int n, int p, float pn, int k,
+                                              const int* er, bool on, int ll, int lw, int& kw) {
   FxAcc nn{0, 0};
   int top = -1000;
   if (on)
@@ -243,18 +245,19 @@ __device__ __forceinline__ long long fx_pivot(const FxMem<SH>& W, int4* Pw, int 
     N += __shfl_xor_sync(0xffffffffu, N, o);
     top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
   }
-  kw = (107 - top) >> 1;
+  kw = fx_pivot_weight(top, pn);
   if (on)
 #pragma unroll 1
     for (int i = ll; i < m; i += lw) Pw[i] = fx_shift_any(W.ld(i * n + p), 2 * er[i] + kw);
   return N;
 }
 
-// Column c of step j (pivot p, y = 1 / |p|, kx = 2 k - kw) by its group of lanes.
+// Column c of step j (pivot p, y = 1 / |p|, kx = 2 k - kw) by its group of lanes;
+// the high limbs that it leaves are ORed into high.
 template <bool SH>
 __device__ __forceinline__ void fx_qr_column(const FxMem<SH>& W, const FxMem<SH>& X, const int4* Pw, int m, int n,
                                              int p, int c, int xoff, Fx y, int kx, const int* er, bool mine, int lig,
-                                             int lg, int lgm, float* cn) {
+                                             int lg, int lgm, float* cn, int& high) {
   FxAcc re{0, 0}, im{0, 0};
   if (mine)
 #pragma unroll 1
@@ -272,16 +275,44 @@ __device__ __forceinline__ void fx_qr_column(const FxMem<SH>& W, const FxMem<SH>
       fx_cmac(ur, ui, s, W.ld(i * n + p));
       const int4 b = fx_pack(fx_val(fx_re(a)) + fx_sum(ur), fx_val(fx_im(a)) + fx_sum(ui));
       W.st(i * n + c, b);
+      high |= fx_high_bits(b.x) | fx_high_bits(b.z);
       q = fmaf(fx_cabs2f(b), fx_pow2f(2 * er[i]), q);
     }
   q = fx_group_sum(q, lg, lgm);
   if (mine && lig == 0) cn[c] = q;
 }
 
+// Rows whose entries have passed 2^55 in the columns from position u0 on are taken
+// down, with their exponents, by lw lanes.  Rows of small weight grow when the
+// pivots, chosen by the large rows, are nearly parallel in the small ones: by up
+// to 50 in 64 x 64 thetas of states whose Schmidt values spread over decades, by 128
+// in a Hadamard matrix with one small row; two limbs hold 32.
+template <bool SH>
+__device__ __noinline__ void fx_rescale_rows(FxMem<SH> W, int m, int n, int u0, const int* ord, int* er, bool on, int ll,
+                                             int lw) {
+  if (on)
+#pragma unroll 1
+    for (int i = ll; i < m; i += lw) {
+      int high = 0;
+#pragma unroll 1
+      for (int u = u0; u < n; ++u) {
+        const int4 a = W.ld(i * n + ord[u]);
+        high |= fx_high_bits(a.x) | fx_high_bits(a.z);
+      }
+      const int k = fx_row_shift(high);
+      if (k > 0) {
+#pragma unroll 1
+        for (int u = u0; u < n; ++u) W.st(i * n + ord[u], fx_shift(W.ld(i * n + ord[u]), -k));
+        er[i] += k;
+      }
+    }
+}
+
 static __device__ __noinline__ int fx_qr(double2* T, int4* Pw, int m, int n, double fro, int4* Xp, int ldx, int* xe,
                                          int* ord, float* cn, int* er, int lane, int lw) {
   const FxMem<true> W(reinterpret_cast<int4*>(T)), X(Xp);
   const int ll = lane & (lw - 1);
+  const unsigned hmask = lw == 32 ? 0xffffffffu : (0xffffu << (lane & 16));
   int xmax = -2000;
   {
     const int lg = fx_lanes(m, lw), gi = ll >> lg, lig = ll & ((1 << lg) - 1), groups = lw >> lg;
@@ -337,7 +368,7 @@ static __device__ __noinline__ int fx_qr(double2* T, int4* Pw, int m, int n, dou
     const int up = on ? 127 - (int)(key & 127u) : 0;
     const int p = on ? ord[up] : 0, k = on ? fx_pivot_shift(pn) : 0;
     int kw;
-    const long long N = fx_pivot(W, Pw, m, n, p, k, er, on, ll, lw, kw);
+    const long long N = fx_pivot(W, Pw, m, n, p, pn, k, er, on, ll, lw, kw);
     if (on && ll == 0) {   // every lane has read ord[up] (the shuffles above)
       ord[up] = ord[j];
       ord[j] = p;
@@ -353,13 +384,19 @@ static __device__ __noinline__ int fx_qr(double2* T, int4* Pw, int m, int n, dou
     const int na = on ? n - j - 1 : 0;
     const int lg = fx_lanes(na, lw), gi = ll >> lg, lig = ll & ((1 << lg) - 1), groups = lw >> lg;
     const int iters = fx_umax((na + groups - 1) / groups), lgm = fx_umax(lg);
+    int high = 0;
 #pragma unroll 1
     for (int it = 0; it < iters; ++it) {
       const int u = j + 1 + gi + it * groups;
       const bool mine = on && u < n;
-      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, 2 * k - kw, er, mine, lig, lg, lgm, cn);
+      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, 2 * k - kw, er, mine, lig, lg, lgm, cn, high);
     }
     __syncwarp();
+    const unsigned grown = __ballot_sync(0xffffffffu, high >= (1 << 27));
+    if (grown != 0u) {
+      fx_rescale_rows(W, m, n, j + 1, ord, er, on && (grown & hmask) != 0u, ll, lw);
+      __syncwarp();
+    }
   }
   return rank;
 }
@@ -432,7 +469,7 @@ __device__ __noinline__ int fx_qr_cta(double2* T, int4* Pw, int m, int n, double
       const int up = 127 - (int)(key & 127u);
       const int p = on ? ord[up] : -1, k = on ? fx_pivot_shift(pn) : 0;
       int kw;
-      const long long N = fx_pivot(W, Pw, m, n, p, k, er, on, ti, 32, kw);
+      const long long N = fx_pivot(W, Pw, m, n, p, pn, k, er, on, ti, 32, kw);
       if (ti == 0) {
         if (on) {
           ord[up] = ord[j];
@@ -459,13 +496,17 @@ __device__ __noinline__ int fx_qr_cta(double2* T, int4* Pw, int m, int n, double
     for (int u = ti; u < j; u += nt) X.st(j * ldx + ord[u], make_int4(0, 0, 0, 0));
     const int na = n - j - 1;
     const int lg = fx_cta_lanes(na), gi = ti >> lg, lig = ti & ((1 << lg) - 1), groups = nt >> lg;
+    int high = 0;
 #pragma unroll 1
     for (int u0 = j + 1; u0 < n; u0 += groups) {
       const int u = u0 + gi;
       const bool mine = u < n;
-      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, kx, er, mine, lig, lg, lg, cn);
+      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, kx, er, mine, lig, lg, lg, cn, high);
     }
-    __syncthreads();
+    if (__syncthreads_or(high >= (1 << 27))) {
+      fx_rescale_rows(W, m, n, j + 1, ord, er, true, ti, nt);
+      __syncthreads();
+    }
   }
   return own;
 }
