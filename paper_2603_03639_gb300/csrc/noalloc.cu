@@ -126,7 +126,7 @@ extern "C" tnrc_status tnrc_fidelity_static(const tnrc_problem* pb, const tnrc_m
   int maxb = 0;
   for (int par = 0; par < 2; ++par) maxb = std::max(maxb, (N - 1 - par + 1) / 2);
   const int warps = std::max(2, std::min(tnrc::kWarps, maxb));
-  const int slab = std::min(1024, d * d * chi * chi);
+  const int slab = std::min(1024, tnrc_host::slab_need(dcap, d));
   const int64_t cc = (int64_t)chi * chi;
   const int64_t scratch_elems = (4 * (int64_t)d * d + d) * cc;   // the same per-warp layout as tnrc_create
   const int64_t env_elems = 2 * (int64_t)(N + 1) * cc;

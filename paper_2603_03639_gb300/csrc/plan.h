@@ -78,6 +78,22 @@ struct Plan {
       off_owner, total;
 };
 
+// Complex elements of shared slab that a warp can use at bonds of full dimension:
+// an update (theta, R^dagger, a pivot column and Phi: upd_elems of traj_impl.cuh),
+// two side by side where bonds go in pairs (from 33 sites on), or the costate's
+// product with the gradient's intermediates.
+inline int slab_need(const std::vector<int>& dcap, int d) {
+  const int N = (int)dcap.size() - 1;
+  int need = 0;
+  for (int b = 0; b + 2 <= N; ++b) {
+    const int m = d * dcap[b], n = d * dcap[b + 2], dl = dcap[b];
+    const int upd = 2 * m * n + std::min(m, n) * (n | 1) + m;
+    const int grad = 2 * m * n + dl * d * dcap[b + 1] + dl * d * d * dcap[b + 2];
+    need = std::max(need, std::max(N >= 33 ? 2 * upd : upd, grad));
+  }
+  return need;
+}
+
 inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan& P, bool limit_by_memory) {
   if (!pb || pb->struct_size != sizeof(tnrc_problem)) return false;
   const int N = pb->n_sites, K = pb->n_slices, chi = pb->chi_max;
@@ -160,14 +176,17 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
   const int ctas_per_sm =
       std::max(1, std::min(pb->ctas_per_sm > 0 ? pb->ctas_per_sm : two ? 2 : 1, (P.d == 4 ? 1 : 2) * tnrc::kWarps / P.warps));
   P.min_blocks = (P.warps * ctas_per_sm > tnrc::kWarps) ? 2 : 1;
-  // each warp's shared slab holds theta^dagger up to slab_elems complex values
-  // (wider thetas use global scratch): split what the resident CTAs of an SM
-  // leave after the per-warp arrays, within the 227 KB a CTA may use
+  // each warp's shared slab: what the resident CTAs of an SM leave after the
+  // per-warp arrays, within the 227 KB a CTA may use, but no more than its bonds need
+  // (the rest serves as L1: 8 qubits at chi = 16 take 4.06 ms with the 1024 elements
+  // they need and 4.20 with 1472).  Wider updates go to the whole CTA: with room for
+  // theta alone every full bond did, and 152 trajectories of 30 qubits at chi = 8 took
+  // 358 ms, 125 with room for the update.
   {
     const int per_sm = 220 * 1024 / ctas_per_sm;
     const int small = (int)tnrc_traj_smem(P.warps, 0) + 1024;
     const int per_warp = std::max(0, per_sm - small) / P.warps / 16;
-    P.slab_elems = std::max(256, std::min(P.d * P.d * chi * chi, per_warp / 32 * 32));
+    P.slab_elems = std::max(256, std::min(slab_need(P.dcap, P.d), per_warp / 32 * 32));
   }
   const int64_t cc = (int64_t)chi * chi;
   // per warp: Phi (d chi)^2, theta (d chi)^2, then the gradient's three
