@@ -99,9 +99,10 @@ typedef struct {
   int32_t ctas_per_sm;           /* resident trajectory CTAs per SM, 1..4, clamped to
                                     warps_per_cta * ctas_per_sm <= 16; above 8 warps per SM
                                     the kernel's 128-register build runs; 0 = 1, or 2 CTAs of
-                                    4 warps when both are 0, the trajectories fill them, their
-                                    work regions take at most 32 GiB and (operators) half of
-                                    an SM's shared memory holds the largest theta           */
+                                    4 warps when both are 0, there are more trajectories than
+                                    SMs, their work regions take at most 32 GiB and
+                                    (operators) half of an SM's shared memory holds the
+                                    largest theta                                           */
   int32_t crosstalk_terms;       /* 1 (or 0): J^z ZZ per bond, J[M][N-1]; 3: the Heisenberg
                                     type J^x XX + J^y YY + J^z ZZ of Eq. Hp, J[M][N-1][3]
                                     in the order (x, y, z)                                 */

@@ -146,18 +146,23 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
   P.warps = tnrc::kWarps;
   if (pb->warps_per_cta < 0 || pb->warps_per_cta == 1 || pb->warps_per_cta > tnrc::kWarps) return false;
   if (pb->ctas_per_sm < 0 || pb->ctas_per_sm > 4) return false;
-  // two CTAs of half the warps once the trajectories fill them: each CTA's
-  // serial stretches (environment sweeps, layer barriers) then run beside the
-  // other's updates (cnot50 near the solution, 304 trajectories: 479 ms as 8
-  // x 1, 386 ms as 4 x 2; with 152 trajectories of ghz30, 172 and 233 ms).
+  // two CTAs of half the warps as soon as one per SM does not hold the trajectories:
+  // those beyond the SMs then run beside the first instead of after them, and each
+  // CTA's serial stretches (environment sweeps, layer barriers) beside the other's
+  // updates.  ms as 8 x 1 and as 4 x 2, by trajectories:
+  //              152          156          304          340          456
+  //   x50        19.4  24.8   32.8  25.1   36.4  27.1   50.1  47.6   52.8  50.2
+  //   ghz30      16.8  23.3   32.0  25.0   33.4  26.5   48.7  50.3   49.7  51.1
+  //   12 qubits   3.9   4.3    6.5   4.5    7.5   5.2   10.3   9.2   11.2   9.6
+  // (16 slices, gradient; 12 slices on 12 qubits.)
   // Not where the second set of work regions would take tens of GB: a default
   // leaves room for other contexts (a caller can still ask for it).
   // Nor for operators whose largest theta and R^dagger leave half of an SM's
   // shared memory: their bonds do reach the cap, and the CTA then works on them
   // in global scratch (chi 16, 300 trajectories: 4 sites 16.5 ms as 8 x 1 and
   // 12.5 as 4 x 2, 8 sites 379 and 657; 5 sites, 600 trajectories: 77 and 59).
-  bool two = pb->warps_per_cta == 0 && pb->ctas_per_sm == 0 && 2 * T >= 3ll * n_sm &&
-             2ll * n_sm * (2 + P.nseg + P.seg) * P.L.bytes <= (32ll << 30);
+  bool two = pb->warps_per_cta == 0 && pb->ctas_per_sm == 0 && T > n_sm &&
+             std::min<long long>(T, 2ll * n_sm) * (2 + P.nseg + P.seg) * P.L.bytes <= (32ll << 30);
   if (two && P.d == 4) {
     const long long half = (110 * 1024 - (int)tnrc_traj_smem(tnrc::kWarps / 2, 0) - 1024) / 16;
     for (int b = 0; b + 2 <= N; ++b) {

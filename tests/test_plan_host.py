@@ -76,3 +76,20 @@ def test_slab_holds_the_updates_that_the_shared_memory_can(plan, N, operator, sh
             need = max(need, 2 * upd if N >= 33 else upd, 2 * m * n + D[b] * d * D[b + 1] + D[b] * d * d * D[b + 2])
         p = plan(N, 10, chi, 8, operator=operator, warps=shape[0], ctas=shape[1])
         assert p["slab"] == max(256, min(need, left))
+
+
+@pytest.mark.parametrize("N,K,chi,operator", [(50, 16, 32, 0), (30, 16, 64, 0), (12, 12, 32, 0), (4, 8, 16, 1)])
+def test_two_ctas_per_sm_from_one_trajectory_more_than_sms(plan, N, K, chi, operator):
+    for T, shape in ((1, (8, 1)), (152, (8, 152)), (153, (4, 153)), (304, (4, 304)), (1000, (4, 304))):
+        p = plan(N, K, chi, T, operator=operator)
+        assert (p["warps"], p["grid"]) == shape
+
+
+def test_one_cta_per_sm_where_two_take_tens_of_gb(plan):
+    p = plan(50, 100, 64, 256, 8)
+    assert (p["warps"], p["grid"]) == (8, 152)
+    assert plan(50, 100, 64, 256, 8, warps=4, ctas=2)["grid"] == 304   # unless asked for
+
+
+def test_operators_that_need_half_an_sm_keep_one_cta(plan):
+    assert plan(8, 8, 16, 300, operator=1)["warps"] == 8
