@@ -170,29 +170,31 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
       two = two && m * n + std::min(m, n) * (n | 1) + m <= half;
     }
   }
-  if (two) P.warps = tnrc::kWarps / 2;
-  if (pb->warps_per_cta > 0) P.warps = pb->warps_per_cta;
-  if (const char* e = getenv("TNRC_WARPS")) {
-    const int w = atoi(e);
-    if (w >= 2 && w <= tnrc::kWarps) P.warps = w;
-  }
-  // the register file holds 8 warps of the 255-register build per SM and 16 of
-  // the 128-register build; more than 8 warps per SM select the latter
-  const int ctas_per_sm =
-      std::max(1, std::min(pb->ctas_per_sm > 0 ? pb->ctas_per_sm : two ? 2 : 1, (P.d == 4 ? 1 : 2) * tnrc::kWarps / P.warps));
-  P.min_blocks = (P.warps * ctas_per_sm > tnrc::kWarps) ? 2 : 1;
-  // each warp's shared slab: what the resident CTAs of an SM leave after the
-  // per-warp arrays, within the 227 KB a CTA may use, but no more than its bonds need
-  // (the rest serves as L1: 8 qubits at chi = 16 take 4.06 ms with the 1024 elements
-  // they need and 4.20 with 1472).  Wider updates go to the whole CTA: with room for
-  // theta alone every full bond did, and 152 trajectories of 30 qubits at chi = 8 took
-  // 358 ms, 125 with room for the update.
-  {
+  int ctas_per_sm = 1;
+  auto shape = [&]() {
+    P.warps = two ? tnrc::kWarps / 2 : tnrc::kWarps;
+    if (pb->warps_per_cta > 0) P.warps = pb->warps_per_cta;
+    if (const char* e = getenv("TNRC_WARPS")) {
+      const int w = atoi(e);
+      if (w >= 2 && w <= tnrc::kWarps) P.warps = w;
+    }
+    // the register file holds 8 warps of the 255-register build per SM and 16 of
+    // the 128-register build; more than 8 warps per SM select the latter
+    ctas_per_sm = std::max(
+        1, std::min(pb->ctas_per_sm > 0 ? pb->ctas_per_sm : two ? 2 : 1, (P.d == 4 ? 1 : 2) * tnrc::kWarps / P.warps));
+    P.min_blocks = (P.warps * ctas_per_sm > tnrc::kWarps) ? 2 : 1;
+    // each warp's shared slab: what the resident CTAs of an SM leave after the
+    // per-warp arrays, within the 227 KB a CTA may use, but no more than its bonds need
+    // (the rest serves as L1: 8 qubits at chi = 16 take 4.06 ms with the 1024 elements
+    // they need and 4.20 with 1472).  Wider updates go to the whole CTA: with room for
+    // theta alone every full bond did, and 152 trajectories of 30 qubits at chi = 8 took
+    // 358 ms, 125 with room for the update.
     const int per_sm = 220 * 1024 / ctas_per_sm;
     const int small = (int)tnrc_traj_smem(P.warps, 0) + 1024;
     const int per_warp = std::max(0, per_sm - small) / P.warps / 16;
     P.slab_elems = std::max(256, std::min(slab_need(P.dcap, P.d), per_warp / 32 * 32));
-  }
+  };
+  shape();
   const int64_t cc = (int64_t)chi * chi;
   // per warp: Phi (d chi)^2, theta (d chi)^2, then the gradient's three
   // intermediates (at most (d + 2 d^2) chi^2) or the R^dagger of a wide update
@@ -200,12 +202,17 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
   P.scratch_elems = (4 * (int64_t)P.d * P.d + P.d) * cc;
   P.env_elems = 2 * (int64_t)(N + 1) * cc;
   P.work_stride = (int64_t)(2 + P.nseg + P.seg) * P.L.bytes;
-  const int64_t per_cta = P.work_stride + (P.scratch_elems * P.warps + P.env_elems) * 16;
-  int grid = (int)std::min<long long>(T, (long long)n_sm * ctas_per_sm);
-  if (const char* e = getenv("TNRC_GRID")) {
-    const int g = atoi(e);
-    if (g >= 1) grid = (int)std::min<long long>(T, g);
-  }
+  int64_t per_cta = 0;
+  int grid = 0;
+  auto regions = [&]() {
+    per_cta = P.work_stride + (P.scratch_elems * P.warps + P.env_elems) * 16;
+    grid = (int)std::min<long long>(T, (long long)n_sm * ctas_per_sm);
+    if (const char* e = getenv("TNRC_GRID")) {
+      const int g = atoi(e);
+      if (g >= 1) grid = (int)std::min<long long>(T, g);
+    }
+  };
+  regions();
   // fixed parts
   int64_t off = 0;
   auto take = [&](int64_t bytes) {
@@ -237,6 +244,11 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
   const int64_t fixed = off;
   if (limit_by_memory && free_bytes > 0) {
     const int64_t budget = (int64_t)(free_bytes * 0.85) - fixed;
+    if (two && budget / per_cta < grid) {   // the second set of regions does not fit: one CTA with all warps
+      two = false;
+      shape();
+      regions();
+    }
     if (budget < per_cta) return false;
     grid = (int)std::min<int64_t>(grid, budget / per_cta);
   }

@@ -89,9 +89,15 @@ class Request:
         return {"crosstalk": self.crosstalk, "order": self.order, "substeps": self.substeps,
                 "operator": self.operator}
 
-    def footprint(self):
+    def footprint(self, **shape):
         return footprint(self.N, self.K, self.dt, self.chi, self.M, self.C, self.P, cutoff=self.cutoff,
-                         mask=self.mask, **self.form())
+                         mask=self.mask, **self.form(), **shape)
+
+    def shape(self, share):
+        """Context keywords of the launch shape: the default where its context
+        fits ``share`` bytes, else one CTA per SM, which holds half the work
+        regions of the default's two."""
+        return {} if self.footprint() <= share else {"warps": 8, "ctas_per_sm": 1}
 
 
 class _Slot:
@@ -102,17 +108,17 @@ class _Slot:
     its trajectories ends; the slot owns a high- and a low-priority stream
     and runs each request on the one its problem's size calls for."""
 
-    def __init__(self, req: Request, device):
+    def __init__(self, req: Request, device, shape):
         import torch
         self.key = req.key
         lo, hi = torch.cuda.Stream.priority_range() if hasattr(torch.cuda.Stream, "priority_range") else (0, -1)
         self.streams = (torch.cuda.Stream(device=device, priority=hi), torch.cuda.Stream(device=device, priority=lo))
         self.stream = self.streams[1]
         self.ctx = Context(req.N, req.K, req.dt, req.chi, req.M, req.C, req.inputs, req.targets,
-                           cutoff=req.cutoff, mask=req.mask, stream=self.stream.cuda_stream, **req.form())
+                           cutoff=req.cutoff, mask=req.mask, stream=self.stream.cuda_stream, **req.form(), **shape)
         self.ctx.set_pooled(True)   # other requests' CTAs can start between this one's trajectories
         self.ctx.set_graphs(True)   # each request replays the context's captured evaluation
-        self.bytes = req.footprint()
+        self.bytes = req.footprint(**shape)
         self.F = torch.zeros(1, dtype=torch.float64, device=device)
         self.g = torch.zeros((req.K, req.C, req.N), dtype=torch.float64, device=device)
         self.ev0 = torch.cuda.Event(enable_timing=True)
@@ -155,8 +161,10 @@ class Server:
     """Continuous-batching server on one device.
 
     mem_budget: device bytes the resident contexts may hold (default: 60% of
-    the free memory at start); max_inflight: requests on the device at once
-    (short requests may exceed it, up to four times);
+    the free memory at start; a context that takes more than an equal share of
+    it, mem_budget / max_inflight, runs one CTA per SM, with half the work
+    regions); max_inflight: requests on the device at once (short requests may
+    exceed it, up to four times);
     short_s: a request whose problem has been served in at most this many
     seconds of device time runs on a high-priority stream, so that its CTAs
     start before the pending CTAs of longer requests (shortest work first at
@@ -271,7 +279,8 @@ class Server:
         if idle:
             slot = idle[0]
         else:
-            need = req.footprint()
+            shape = req.shape(self.mem_budget // self.max_inflight)
+            need = req.footprint(**shape)
             if need > self.mem_budget:
                 req.error = "request footprint %d B exceeds the server budget %d B" % (need, self.mem_budget)
                 req.finish = time.perf_counter()
@@ -287,7 +296,7 @@ class Server:
                 self.slots.remove(victim)
             import torch
             with torch.cuda.device(self.device):
-                slot = _Slot(req, self.device)
+                slot = _Slot(req, self.device, shape)
             self.slots.append(slot)
         req.start = time.perf_counter()
         t = self._service(req.key)

@@ -93,3 +93,18 @@ def test_one_cta_per_sm_where_two_take_tens_of_gb(plan):
 
 def test_operators_that_need_half_an_sm_keep_one_cta(plan):
     assert plan(8, 8, 16, 300, operator=1)["warps"] == 8
+
+
+def test_two_ctas_per_sm_only_where_their_regions_fit(plan):
+    """Where the free memory limits the CTAs, one CTA with all warps per SM takes the
+    regions that fit; a problem that fits so is not refused."""
+    args = (50, 64, 32, 128, 8)
+    full = plan(*args)
+    assert (full["warps"], full["grid"]) == (4, 304)
+    one = plan(*args, warps=8, ctas=1)
+    assert one["grid"] == 152 and one["gb"] < 0.6 * full["gb"]
+    for free, warps, grid in ((1.3 * full["gb"], 4, 304), (1.1 * full["gb"], 8, 152), (1.3 * one["gb"], 8, 152)):
+        p = plan(*args, free=free)
+        assert (p["warps"], p["grid"]) == (warps, grid)
+    few = plan(*args, free=0.7 * one["gb"])
+    assert few["warps"] == 8 and 0 < few["grid"] < 152
