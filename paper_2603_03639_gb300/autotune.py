@@ -4,7 +4,7 @@ The kernel runs one trajectory per CTA; within a CTA the warps share the
 disjoint bonds of a TEBD layer.  The free choices are the warps per CTA (how
 many bonds of a layer run at once, and how evenly a layer's bonds divide
 among them), the resident CTAs per SM (how many trajectories interleave on an
-SM; the register file holds 8 of this kernel's warps per SM) and the matrix
+SM; above 8 warps per SM the kernel's 128-register build runs) and the matrix
 shape (two small SVDs per warp on the half-warps, or one SVD per warp).  The
 tuner times each candidate on the actual problem with CUDA events around the
 kernel and caches the fastest per shape bucket in a JSON file.
@@ -40,20 +40,31 @@ def load(path=None):
         return {}
 
 
-def lookup(N, K, chi, M, P, C, grad=True, path=None, operator=False):
-    """(warps_per_cta, ctas_per_sm) cached for this shape -- or for the same
-    shape with the nearest ensemble-size bucket -- else (0, 0) (defaults)."""
+N_SM = 152   # a GB300's SMs: ensembles up to here fill one CTA per SM, larger ones want two (csrc/plan.h)
+
+
+def _entry(N, K, chi, M, P, C, grad=True, path=None, operator=False):
+    """The cached entry of this shape, or of the same shape with the nearest
+    ensemble-size bucket, among entries tuned on the same side of N_SM
+    trajectories; None without one.  An entry's ensemble is its
+    "trajectories", or its bucket's size where that is not recorded."""
     cache = load(path)
-    key = shape_key(N, K, chi, M, P, C, grad, operator)
-    e = cache.get(key)
-    if e is None:
-        head, tail = key.split("-T")
-        rest = tail.split("-", 1)[1]
-        t = int(tail.split("-", 1)[0])
-        near = [(abs(np.log2(int(k.split("-T")[1].split("-")[0])) - np.log2(t)), k) for k in cache
-                if k.startswith(head + "-T") and k.split("-T")[1].split("-", 1)[1] == rest]
-        if near:
-            e = cache[min(near)[1]]
+    head, tail = shape_key(N, K, chi, M, P, C, grad, operator).split("-T")
+    t, rest = tail.split("-", 1)
+    near = []
+    for k, e in cache.items():
+        if not k.startswith(head + "-T") or k.split("-T")[1].split("-", 1)[1] != rest:
+            continue
+        bucket = int(k.split("-T")[1].split("-", 1)[0])
+        if (int(e.get("trajectories", bucket)) > N_SM) == (M * P > N_SM):
+            near.append((abs(np.log2(bucket) - np.log2(int(t))), k))
+    return cache[min(near)[1]] if near else None
+
+
+def lookup(N, K, chi, M, P, C, grad=True, path=None, operator=False):
+    """(warps_per_cta, ctas_per_sm) cached for this shape (see _entry), else
+    (0, 0) (defaults)."""
+    e = _entry(N, K, chi, M, P, C, grad, path, operator)
     return (int(e["warps"]), int(e["ctas_per_sm"])) if e else (0, 0)
 
 
@@ -61,13 +72,7 @@ def lookup_pairs(N, K, chi, M, P, C, grad=True, path=None, operator=False):
     """The cached matrix shape for this problem: True = two small SVDs per warp
     on the half-warps (also the default when nothing is cached), False = one
     SVD per warp."""
-    cache = load(path)
-    key = shape_key(N, K, chi, M, P, C, grad, operator)
-    e = cache.get(key)
-    if e is None:
-        w, c = lookup(N, K, chi, M, P, C, grad, path, operator)
-        e = next((v for v in cache.values() if v.get("warps") == w and v.get("ctas_per_sm") == c
-                  and v.get("operator", False) == operator), None)
+    e = _entry(N, K, chi, M, P, C, grad, path, operator)
     return bool(e.get("pairs", True)) if e else True
 
 
@@ -80,7 +85,6 @@ def tune(N, K, dt, chi, M, C, inputs, targets, u, noise, mask=None, grad=True, c
     from .tnrc import Context
     seed, dist, scale = noise
     form = form or {}
-    nb = max((N - 1 + 1) // 2, 1)
     max_warps_per_sm = 8 if form.get("operator") else 16   # operators run the 255-register build only
     times = {}
 
@@ -98,7 +102,7 @@ def tune(N, K, dt, chi, M, C, inputs, targets, u, noise, mask=None, grad=True, c
             times[(w, c, pairs)] = st["traj_ms"] / max(1, st["traj_launches"])
 
     for w, c in candidates:
-        if w * c > max_warps_per_sm or w > max(2, nb):
+        if w * c > max_warps_per_sm:   # every warp count: they share the large bonds and the environments
             continue
         run(w, c, True)
     for w, c, _ in sorted(times, key=times.get)[:2]:
@@ -132,7 +136,7 @@ def main():
     key = shape_key(w.N, w.K, w.chi, w.M, w.P, w.C, grad, w.operator)
     name = lambda k: "%dx%d%s" % (k[0], k[1], "" if k[2] else "-warp")  # noqa: E731
     cache[key] = {"warps": best[0], "ctas_per_sm": best[1], "pairs": bool(best[2]), "workload": w.name,
-                  "operator": bool(w.operator), "ms": {name(k): round(v, 3) for k, v in times.items()}}
+                  "operator": bool(w.operator), "trajectories": w.M * w.P, "ms": {name(k): round(v, 3) for k, v in times.items()}}
     with open(args.out, "w") as f:
         json.dump(cache, f, indent=1, sort_keys=True)
     print(json.dumps({"key": key, "best": name(best), "ms": {name(k): v for k, v in times.items()}}))
