@@ -672,12 +672,15 @@ __device__ __forceinline__ double2* env_right(const TrajParams& p, int region) {
 }
 
 // The team of one sweep meets at its named barrier; a single warp (team < 0)
-// needs none.
+// needs none.  Literal barrier numbers: with one in a register the kernel is given
+// all 16.
 __device__ __forceinline__ void team_sync(int team, int nt) {
   if (team < 0)
     __syncwarp();
+  else if (team == 0)
+    asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
   else
-    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(nt) : "memory");
+    asm volatile("bar.sync 2, %0;" ::"r"(nt) : "memory");
 }
 
 // One step by thread ti of nt, in FP64.  Left (team 0, or one warp with team -1):
