@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(kGateThreads) layer_gate_kernel(LayerGateArgs 
     for (int j = 1; j < 4; ++j)
       if (j == r) lam = h[j].x;
     double sn, cs;
-    sincos(tau * lam, &sn, &cs);
-    const double2 E = make_double2(cs, -sn);   // e^{-i tau lam_r}
+    sincos(0.5 * tau * lam, &sn, &cs);
+    const double2 E = make_double2(-2.0 * sn * sn, -2.0 * sn * cs);   // e^{-i tau lam_r} - 1
     double2 ge[4], vE[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -316,10 +316,13 @@ __global__ void __launch_bounds__(kGateThreads) layer_gate_kernel(LayerGateArgs 
     __syncwarp();
     if (mine) {
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {   // G = V E V^dagger
+      for (int cc = 0; cc < 4; ++cc) {
+        // G = 1 + V (E - 1) V^dagger: what V lacks in orthogonality (some 1e-16, the
+        // roundings of its rotations) then enters times the angle and not times one
         double2 g = make_double2(0.0, 0.0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) cfmac(g, S.V[f][cc * 4 + j], vE[j]);
+        if (cc == r) g.x += 1.0;
         S.G[f][r * 4 + cc] = g;
       }
     }
