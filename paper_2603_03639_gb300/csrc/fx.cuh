@@ -48,6 +48,22 @@ TNRC_HD void fx_mac(FxAcc& s, Fx a, Fx b) {
 // the sum / 2^56, rounded
 TNRC_HD long long fx_sum(FxAcc s) { return s.h + ((s.x + (1ll << 27)) >> 28); }
 
+// the sum / 2^(56 - sh), rounded, 0 <= sh < 28
+TNRC_HD long long fx_sum_shifted(FxAcc s, int sh) { return (s.h << sh) + ((s.x + (1ll << (27 - sh))) >> (28 - sh)); }
+
+// A sum of squares h 2^56 + 2 x 2^28 + l, and itself / 2^56, rounded.  The low parts
+// are all positive here: dropped, they would bias a norm by a sixth of a unit of
+// 2^-56 an entry.
+struct FxSquares {
+  long long h, x, l;
+};
+TNRC_HD void fx_square(FxSquares& s, Fx a) {
+  s.h += (long long)a.hi * a.hi;
+  s.x += (long long)a.hi * a.lo;
+  s.l += (long long)a.lo * a.lo;
+}
+TNRC_HD long long fx_sum(FxSquares s) { return s.h + ((s.x + (s.l >> 29) + (1ll << 26)) >> 27); }
+
 TNRC_HD long long fx_mul(Fx a, Fx b) {
   FxAcc s{0, 0};
   fx_mac(s, a, b);
@@ -135,12 +151,19 @@ TNRC_HD int fx_row_shift(int high_bits) {
 }
 
 // The exponent kw of a pivot column's weighted copy, p_i 2^(2 er_i + kw): entries
-// below 2^54 (top: the largest log2 |p_i 2^(2 er_i)|^2), and inner products with the
+// below 2^56 (top: the largest log2 |p_i 2^(2 er_i)|^2), and inner products with the
 // remaining columns, which |p|^2 2^kw bounds (pn = |p|^2, the largest left), below
-// 2^(56 + 58).
+// 2^(56 + 57).  They are kept as multiples of 2^(56 - sh), sh = fx_dot_shift, so that
+// an inner product near the bound has 57 bits whatever the columns' shape.  As large
+// as both allow: the low x low products that fx_mac drops are up to 2^54 each, and
+// beside |p|^2 2^kw they are what is lost.
 TNRC_HD int fx_pivot_weight(int top, float pn) {
-  const int a = (107 - top) >> 1, b = 113 - fx_ilog2f(pn);
+  const int a = (111 - top) >> 1, b = 112 - fx_ilog2f(pn);
   return a < b ? a : b;
+}
+TNRC_HD int fx_dot_shift(int kw, float pn) {
+  const int sh = 112 - fx_ilog2f(pn) - kw;
+  return sh < 27 ? sh : 27;
 }
 
 // 1 / sqrt(N 2^-56) in units of 2^-56, for N in about [2^54, 2^56]: the float

@@ -228,18 +228,20 @@ __device__ __forceinline__ unsigned fx_pivot_key(const float* cn, const int* ord
 template <bool SH>
 __device__ __forceinline__ long long fx_pivot(const FxMem<SH>& W, int4* Pw, int m, int n, int p, float pn, int k,
                                               const int* er, bool on, int ll, int lw, int& kw) {
-  FxAcc nn{0, 0};
+  FxSquares nn{0, 0, 0};
   int top = -1000;
   if (on)
 #pragma unroll 1
     for (int i = ll; i < m; i += lw) {
       const int4 a = W.ld(i * n + p);
       const int e = er[i];
-      fx_cabs2(nn, fx_shift_any(a, e + k));
+      const int4 f = fx_shift_any(a, e + k);
+      fx_square(nn, fx_re(f));
+      fx_square(nn, fx_im(f));
       const float q = fx_cabs2f(a);
       if (q > 0.0f) top = max(top, fx_ilog2f(q) + 4 * e);
     }
-  long long N = fx_sum2(nn);
+  long long N = fx_sum(nn);
 #pragma unroll 1
   for (int o = lw >> 1; o > 0; o >>= 1) {
     N += __shfl_xor_sync(0xffffffffu, N, o);
@@ -252,17 +254,19 @@ __device__ __forceinline__ long long fx_pivot(const FxMem<SH>& W, int4* Pw, int 
   return N;
 }
 
-// Column c of step j (pivot p, y = 1 / |p|, kx = 2 k - kw) by its group of lanes;
+// Column c of step j (pivot p, y = 1 / |p|, inner products shifted by sh, kx = 2 k -
+// kw - sh) by its group of lanes;
 // the high limbs that it leaves are ORed into high.
 template <bool SH>
 __device__ __forceinline__ void fx_qr_column(const FxMem<SH>& W, const FxMem<SH>& X, const int4* Pw, int m, int n,
-                                             int p, int c, int xoff, Fx y, int kx, const int* er, bool mine, int lig,
+                                             int p, int c, int xoff, Fx y, int sh, int kx, const int* er, bool mine, int lig,
                                              int lg, int lgm, float* cn, int& high) {
   FxAcc re{0, 0}, im{0, 0};
   if (mine)
 #pragma unroll 1
     for (int i = lig; i < m; i += 1 << lg) fx_cmacc(re, im, Pw[i], W.ld(i * n + c));
-  const long long dr = fx_group_sum(fx_sum(re), lg, lgm), di = fx_group_sum(fx_sum(im), lg, lgm);
+  const long long dr = fx_group_sum(fx_sum_shifted(re, sh), lg, lgm);
+  const long long di = fx_group_sum(fx_sum_shifted(im, sh), lg, lgm);
   const int4 r = fx_shift_any(fx_pack(fx_mul(fx_split(dr), y), fx_mul(fx_split(di), y)), kx);
   if (mine && lig == 0) X.st(xoff + c, make_int4(r.x, r.y, -r.z, -r.w));
   const int4 s = fx_pack(-fx_mul(fx_re(r), y), -fx_mul(fx_im(r), y));
@@ -381,6 +385,7 @@ static __device__ __noinline__ int fx_qr(double2* T, int4* Pw, int m, int n, dou
 #pragma unroll 1
       for (int u = ll; u < j; u += lw) X.st(j * ldx + ord[u], make_int4(0, 0, 0, 0));
     }
+    const int sh = on ? fx_dot_shift(kw, pn) : 0, kx = 2 * k - kw - sh;
     const int na = on ? n - j - 1 : 0;
     const int lg = fx_lanes(na, lw), gi = ll >> lg, lig = ll & ((1 << lg) - 1), groups = lw >> lg;
     const int iters = fx_umax((na + groups - 1) / groups), lgm = fx_umax(lg);
@@ -389,7 +394,7 @@ static __device__ __noinline__ int fx_qr(double2* T, int4* Pw, int m, int n, dou
     for (int it = 0; it < iters; ++it) {
       const int u = j + 1 + gi + it * groups;
       const bool mine = on && u < n;
-      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, 2 * k - kw, er, mine, lig, lg, lgm, cn, high);
+      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, sh, kx, er, mine, lig, lg, lgm, cn, high);
     }
     __syncwarp();
     const unsigned grown = __ballot_sync(0xffffffffu, high >= (1 << 27));
@@ -410,7 +415,7 @@ __device__ __forceinline__ int fx_cta_lanes(int units) {
   return lg > 5 ? 5 : lg;
 }
 struct FxQrShared {
-  int p, k, kw, xmax;
+  int p, sh, kx, xmax;
   long long y, N;
 };
 
@@ -475,8 +480,8 @@ __device__ __noinline__ int fx_qr_cta(double2* T, int4* Pw, int m, int n, double
           ord[up] = ord[j];
           ord[j] = p;
           xe[j] = E0 - k;
-          sh->k = k;
-          sh->kw = kw;
+          sh->sh = fx_dot_shift(kw, pn);
+          sh->kx = 2 * k - kw - sh->sh;
           sh->N = N;
           sh->y = fx_rsqrt(N);
         }
@@ -490,7 +495,7 @@ __device__ __noinline__ int fx_qr_cta(double2* T, int4* Pw, int m, int n, double
       return j;
     }
     const Fx y = fx_split(sh->y);
-    const int kx = 2 * sh->k - sh->kw;
+    const int ds = sh->sh, kx = sh->kx;
     if (ti == 0) X.st(j * ldx + p, fx_pack(fx_mul(fx_split(sh->N), y), 0));
 #pragma unroll 1
     for (int u = ti; u < j; u += nt) X.st(j * ldx + ord[u], make_int4(0, 0, 0, 0));
@@ -501,7 +506,7 @@ __device__ __noinline__ int fx_qr_cta(double2* T, int4* Pw, int m, int n, double
     for (int u0 = j + 1; u0 < n; u0 += groups) {
       const int u = u0 + gi;
       const bool mine = u < n;
-      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, kx, er, mine, lig, lg, lg, cn, high);
+      fx_qr_column(W, X, Pw, m, n, p, mine ? ord[u] : 0, j * ldx, y, ds, kx, er, mine, lig, lg, lg, cn, high);
     }
     if (__syncthreads_or(high >= (1 << 27))) {
       fx_rescale_rows(W, m, n, j + 1, ord, er, true, ti, nt);

@@ -198,11 +198,15 @@ __device__ __noinline__ int theta_rank(const TrajParams& p, const Lay& Y, unsign
 #pragma unroll 1
     for (int c0 = 0; c0 < r; c0 += groups) {
       const int c = c0 + gi;
-      FxAcc nn{0, 0};
+      FxSquares nn{0, 0, 0};
       if (c < r)
 #pragma unroll 1
-        for (int i = lig; i < n; i += 1 << lg) fx_cabs2(nn, X[c * ldx + i]);
-      const long long N = fx_group_sum(fx_sum2(nn), lg, lg);
+        for (int i = lig; i < n; i += 1 << lg) {
+          const int4 a = X[c * ldx + i];
+          fx_square(nn, fx_re(a));
+          fx_square(nn, fx_im(a));
+        }
+      const long long N = fx_group_sum(fx_sum(nn), lg, lg);
       if (c < r && lig == 0) nrm[c].n2 = N;
     }
   }
