@@ -85,7 +85,7 @@ def tune(N, K, dt, chi, M, C, inputs, targets, u, noise, mask=None, grad=True, c
     from .tnrc import Context
     seed, dist, scale = noise
     form = form or {}
-    max_warps_per_sm = 8 if form.get("operator") else 16   # operators run the 255-register build only
+    max_warps_per_sm = 8 if form.get("operator") else 16   # operators have no 128-register build
     times = {}
 
     def run(w, c, pairs):

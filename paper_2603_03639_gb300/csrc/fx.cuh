@@ -2,13 +2,14 @@
 // common power-of-two scale in the place of FP64 values.
 //
 // GB300 issues one warp-wide FP64 FMA per sub-partition every 64 cycles and a
-// 32 x 32 + 64 bit integer multiply-add (IMAD.WIDE) every 2, so a product of
-// two 56-bit numbers as three integer multiply-adds costs a tenth of one DFMA.
+// 32 x 32 + 64 bit integer multiply-add (IMAD.WIDE) about every 5 (both measured),
+// so a product of two 56-bit numbers as three integer multiply-adds costs a quarter
+// of one DFMA.
 // A value v (|v| < 2^59) is held as two limbs, v = hi 2^28 + lo with lo in
 // [-2^27, 2^27); a complex value is an int4 (re.hi, re.lo, im.hi, im.lo), the
-// 16 bytes of a double2.  Products keep hi hi and the two cross terms (lo lo
-// is below 2^-2 of the last place after the shift by 56 bits) and are summed
-// exactly in two 64-bit accumulators, so a sum is rounded once, at its end.
+// 16 bytes of a double2.  Products keep hi hi and the two cross terms and drop
+// lo lo (up to a quarter of the last place after the shift by 56 bits); what is
+// kept is summed exactly in two 64-bit accumulators and rounded once, at its end.
 // Vectors are scaled so that their norm is near 2^56: a rounding is 2^-57 of
 // the norm, against 2^-53 of each element in FP64.
 #pragma once

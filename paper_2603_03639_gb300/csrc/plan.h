@@ -178,8 +178,8 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
       const int w = atoi(e);
       if (w >= 2 && w <= tnrc::kWarps) P.warps = w;
     }
-    // the register file holds 8 warps of the 255-register build per SM and 16 of
-    // the 128-register build; more than 8 warps per SM select the latter
+    // the register file holds 9 warps of the build without a limit (210 registers) and
+    // 16 of the 128-register build; more than 8 warps per SM select the latter
     ctas_per_sm = std::max(
         1, std::min(pb->ctas_per_sm > 0 ? pb->ctas_per_sm : two ? 2 : 1, (P.d == 4 ? 1 : 2) * tnrc::kWarps / P.warps));
     P.min_blocks = (P.warps * ctas_per_sm > tnrc::kWarps) ? 2 : 1;

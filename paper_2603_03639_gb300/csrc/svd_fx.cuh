@@ -69,17 +69,13 @@ __device__ __forceinline__ int4 fx_shift(int4 a, int k) {   // a 2^k
 // a 2^k for any k (what leaves the 64 bits on the right is zero)
 __device__ __forceinline__ int4 fx_shift_any(int4 a, int k) { return fx_shift(a, k < -62 ? -62 : k); }
 
-// FP64 <-> fixed point: x 2^k rounded, and v 2^e
+// x 2^k, and FP64 to fixed point
 __device__ __forceinline__ double fx_scale(double x, int k) {
   const int h = __double2hiint(x), e = (h >> 20) & 2047;
   return (e == 0 || e + k <= 0) ? 0.0 : __hiloint2double(h + (k << 20), __double2loint(x));
 }
 __device__ __forceinline__ int4 fx_from_double2(double2 a, int k) {
   return fx_pack(__double2ll_rn(fx_scale(a.x, k)), __double2ll_rn(fx_scale(a.y, k)));
-}
-__device__ __forceinline__ double fx_to_double(Fx a, int e) { return fx_scale((double)fx_val(a), e); }
-__device__ __forceinline__ double2 fx_to_double2(int4 a, int e) {
-  return make_double2(fx_to_double(fx_re(a), e), fx_to_double(fx_im(a), e));
 }
 
 // Element access: the matrices of a warp are in shared memory (SH, 32-bit

@@ -97,8 +97,8 @@ struct TrajParams {
   int want_grad;
   int warps;                   // warps per CTA
   int phys_dim;                // 2: qubit states; 4: operators as vectors (s = 2 out + in)
-  int min_blocks;              // register budget of the launch: 1 = up to 8 warps per SM
-                               // (255 registers), 2 = up to 16 warps per SM (128 registers)
+  int min_blocks;              // build of the launch: 1 = up to 8 warps per SM (no limit on
+                               // registers), 2 = up to 16 warps per SM (128 registers)
   int slab_elems;              // complex elements of each warp's shared slab
   int cta_slab_elems;          // of all warps' slabs together (contiguous)
   Lay full;                    // capacities min(2^i, 2^(N-i), chi)
@@ -120,7 +120,7 @@ struct TrajParams {
   double2* O;                      // [T]
   double* gsp;                     // [T][K*C*N] or null
   double* disc;                    // [T]
-  unsigned long long* counters;    // see kCtrHist in traj.cu
+  unsigned long long* counters;    // see kCtrHist in traj_impl.cuh
   int* status;
   int* work_counter;
   // launch mode: 0 = persistent (grid <= resident CTAs; each CTA takes
@@ -128,7 +128,7 @@ struct TrajParams {
   // 1 = pooled (one CTA per trajectory, t = blockIdx.x; the CTA holds one of
   // n_regions work regions from region_owner while it runs, so the block
   // scheduler can interleave CTAs of other launches between trajectories)
-  int pair_svd;                    // 1: two small SVDs per warp on the half-warps (see traj.cu)
+  int pair_svd;                    // 1: two small SVDs per warp on the half-warps (traj_impl.cuh)
   int pooled;
   int n_regions;
   int* region_owner;               // [n_regions], 0 = free

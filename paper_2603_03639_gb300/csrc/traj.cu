@@ -28,7 +28,7 @@ extern "C" cudaError_t tnrc_traj_occupancy(int phys_dim, int min_blocks, int war
 
 extern "C" cudaError_t tnrc_launch_traj(const tnrc::TrajParams* p, int grid, size_t smem, cudaStream_t st) {
   (void)cudaGetLastError();  // report only this launch below
-  // operators (physical dimension 4) run the 255-register build only
+  // operators (physical dimension 4) have only the build without a register limit
   if (p->phys_dim == 4) return tnrc_op_launch(p, grid, smem, st);
   if (p->min_blocks == 2)
     tnrc::traj_kernel<2, 2><<<grid, p->warps * 32, smem, st>>>(*p);

@@ -500,11 +500,18 @@ __device__ __noinline__ void wide_update_cta(const TrajParams& p, const Lay& Y, 
 
 constexpr int kPairSide = 64;
 
-// Bonds a warp takes at a time.  Two, with small ones as a pair, where a layer
-// has more bonds than an SM's eight warps twice over; one below that, where
-// pairs would leave warps without a bond (8 qubits, 4 bonds a layer: 5.9 ms
-// two at a time).  By the layer's bonds only, so that results do not depend on
-// the launch.
+// Bonds a warp takes at a time.  Two, with small ones as a pair, on chains of 33
+// sites or more; one below that, where pairs leave warps without a bond (8 qubits,
+// 4 bonds a layer: 5.9 ms two at a time, 4.7 one).  By the layer's bonds only, so
+// that results do not depend on the launch.  ms one / two at a time, gradient, 16
+// slices, 152 trajectories as 8 x 1 and 304 as 4 x 2:
+//            near a solution (bonds to 9)       random controls (bonds to 19)
+//   sites    8 x 1          4 x 2               8 x 1          4 x 2
+//   20        7.6 /  8.7    13.1 / 11.2         13.8 / 17.5    21.0 / 21.9
+//   26       11.0 / 10.0    16.8 / 15.6         15.1 / 15.6    22.4 / 23.7
+//   33       12.9 / 11.4    22.4 / 18.5         17.6 / 18.4    29.9 / 27.9
+//   38       15.8 / 14.5    25.9 / 22.0         21.1 / 20.7    34.4 / 32.8
+//   50       19.2 / 18.5    33.9 / 27.0         27.1 / 28.9    46.7 / 43.5
 __device__ __forceinline__ int group_size(const TrajParams& p) { return p.N - 1 >= 32 ? 2 : 1; }
 
 // Whether bonds b1 and b2 of one layer are updated as a pair: pairing is on
@@ -759,10 +766,12 @@ __device__ __forceinline__ long long update_cost(int Dl, int Dr) {
 // not fit the warp's shared slab, or it is a good part of the layer's work
 // (more than a sixth; one warp would then still be at it when the others are
 // done with the rest) and large enough for its rounds to occupy several warps
-// (echo12_cap, theta up to 64 x 64, 5 or 6 bonds a layer: 661 ms with one warp
-// per bond, 130 ms shared).  The rule looks at sizes only, and the work is cut
-// into the same lane groups whatever the number of warps, so results do not
-// depend on it.
+// (12 qubits at the cap, theta up to 64 x 64, 5 or 6 bonds a layer: 661 ms with one
+// warp per bond, 130 ms shared).  The rule looks at sizes and at the slab, and the
+// work is cut into the same lane groups whatever the number of warps, so for one slab
+// size results depend neither on that nor on what else runs.  Another launch shape or
+// the allocation-free entry point, with another slab, may take a bond on another path:
+// the same up to the order of sums.
 constexpr int kWideSide = 16;
 template <int kD>
 __device__ __forceinline__ bool wide_update(const TrajParams& p, const int* D, int b, long long total) {
@@ -1025,9 +1034,9 @@ __device__ __noinline__ int copy_slot(const TrajParams& p, const Lay& Ys, const 
 
 // Entries e and e+1 of the layer's bond order (w.order, nb entries): one
 // warp updates both, as a pair when both are small (two_site_update_pair),
-// else one after the other.  The grouping depends only on the order and the
-// bond dimensions, not on which warp or CTA takes it, so every launch form
-// computes the same thing.
+// else one after the other.  The grouping depends only on the order, the bond
+// dimensions and the slab, not on which warp or CTA takes it, so every launch form
+// of one shape computes the same thing.
 template <int kD>
 __device__ __noinline__ void forward_group(const TrajParams& p, const Lay& Y, unsigned char* slot, int s, int l, int e, int nb,
                               bool adjoint, bool record, bool count, WarpCtx& w) {
@@ -1270,9 +1279,10 @@ __device__ __noinline__ int run_trajectory(const TrajParams& p, bool packed, uns
   return 0;
 }
 
-// Compiled twice: kMinBlocks = 1 lets a thread use up to 255 registers (at
-// most 8 warps per SM); kMinBlocks = 2 caps it at 128 so that 16 warps fit an
-// SM, trading a few spilled values for twice the warps to hide FP64 latency.
+// Compiled twice: kMinBlocks = 1 without a limit on registers (210 a thread, 208 for
+// operators: nine warps would fit an SM, launches use up to eight); kMinBlocks = 2
+// with at most 128 so that 16 warps fit, trading a few spilled values for twice the
+// warps to hide latency.
 template <int kMinBlocks, int kD>
 __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) traj_kernel(TrajParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
