@@ -353,7 +353,7 @@ def gpu_arm(args, w):
         # per step: noise_kernel, layer_gate_kernel, traj_kernel, reduce_fidelity_kernel,
         # reduce_grad_kernel (the launch list under profiles/ shows the same five)
         "gpu_launches": 5 * args.steps,
-        "launch_shape": {"warps_per_cta": tuned[0] or "default", "ctas_per_sm": tuned[1] or 1,
+        "launch_shape": {"warps_per_cta": tuned[0] or "default", "ctas_per_sm": tuned[1] or "default",
                          "svd": "two per warp (half-warps)" if pairs else "one per warp",
                          "source": "autotune cache" if tuned[0] else "default"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -595,7 +595,8 @@ def plain_arm(args, w):
 
     ws = w.replace(M=args.plain_samples)
     ins, tgs = ws.states()
-    tuned = autotune.lookup(w.N, w.K, w.chi, w.M, w.P, w.C, grad=True, operator=w.operator)
+    # the sample's own shape: that of the full ensemble leaves half the warps idle on a few trajectories
+    tuned = autotune.lookup(ws.N, ws.K, ws.chi, ws.M, ws.P, ws.C, grad=True, operator=ws.operator)
     out, ref = {}, None
     with ClockSampler(int(os.environ.get("LOCAL_RANK", "0"))) as clk:
         for mode in ("batched", "plain", "one_cta"):
@@ -606,8 +607,8 @@ def plain_arm(args, w):
                               mask=ws.mask(), warps=tuned[0], ctas_per_sm=tuned[1], **form_kwargs(ws))
             finally:
                 os.environ.pop("TNRC_GRID", None)
-            ctx.set_svd_shape(autotune.lookup_pairs(w.N, w.K, w.chi, w.M, w.P, w.C, grad=True,
-                                                    operator=w.operator))
+            ctx.set_svd_shape(autotune.lookup_pairs(ws.N, ws.K, ws.chi, ws.M, ws.P, ws.C, grad=True,
+                                                    operator=ws.operator))
             ctx.set_controls(ws.controls())
             ctx.sample_noise(ws.seed_J, ws.noise_dist, ws.noise_scale)
             run = ctx.fidelity_grad_plain if mode == "plain" else ctx.fidelity_grad
@@ -631,7 +632,7 @@ def plain_arm(args, w):
             "speedup_vs_plain": out["batched"]["value"] / out["plain"]["value"],
             "speedup_vs_one_cta": out["batched"]["value"] / out["one_cta"]["value"],
             "results_identical": all(v["identical_to_batched"] for v in out.values()),
-            "launch_shape": {"warps_per_cta": tuned[0] or "default", "ctas_per_sm": tuned[1] or 1},
+            "launch_shape": {"warps_per_cta": tuned[0] or "default", "ctas_per_sm": tuned[1] or "default"},
             "clocks": clk.summary()}
     print(json.dumps(line), flush=True)
 
