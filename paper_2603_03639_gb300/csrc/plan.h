@@ -248,6 +248,11 @@ inline bool make_plan(const tnrc_problem* pb, int n_sm, size_t free_bytes, Plan&
       two = false;
       shape();
       regions();
+      if (budget < per_cta) {   // nor one region of eight warps (their scratch can outweigh the states)
+        two = true;
+        shape();
+        regions();
+      }
     }
     if (budget < per_cta) return false;
     grid = (int)std::min<int64_t>(grid, budget / per_cta);

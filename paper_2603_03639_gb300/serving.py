@@ -95,9 +95,10 @@ class Request:
 
     def shape(self, share):
         """Context keywords of the launch shape: the default where its context
-        fits ``share`` bytes, else one CTA per SM, which holds half the work
-        regions of the default's two."""
-        return {} if self.footprint() <= share else {"warps": 8, "ctas_per_sm": 1}
+        fits ``share`` bytes, else one CTA per SM where that takes less (half the
+        work regions of the default's two, but eight warps' scratch in each)."""
+        one = {"warps": 8, "ctas_per_sm": 1}
+        return {} if self.footprint() <= max(share, self.footprint(**one)) else one
 
 
 class _Slot:

@@ -108,3 +108,14 @@ def test_two_ctas_per_sm_only_where_their_regions_fit(plan):
         assert (p["warps"], p["grid"]) == (warps, grid)
     few = plan(*args, free=0.7 * one["gb"])
     assert few["warps"] == 8 and 0 < few["grid"] < 152
+
+
+def test_a_context_of_four_warps_is_kept_where_eight_do_not_fit(plan):
+    """Short chains at chi = 64: a region is mostly its warps' scratch (1.2 MB each)."""
+    args = (10, 4, 64, 160)
+    fixed = plan(*args)["gb"] - 160 * (plan(*args)["gb"] - plan(*args, warps=4, ctas=1)["gb"]) / 8.0   # without regions
+    four = (plan(*args)["gb"] - fixed) / 160
+    eight = (plan(*args, warps=8, ctas=1)["gb"] - fixed) / 152
+    assert eight > 1.3 * four
+    p = plan(*args, free=(fixed + 0.5 * (four + eight)) / 0.85)
+    assert p is not None and p["warps"] == 4 and p["grid"] == 1
